@@ -3,7 +3,7 @@
 // Sec. 3.1) with the lists cut into windows of lambda ids (Sec. 3.3.1).
 //
 // Pipeline (one stream):
-//   validate_indptr  -> prune_rows (warp per row) [+ prune_long_rows (block per row)]
+//   validate_indptr  -> prune_select (warp per row) [+ prune_rows, prune_long_rows: rows that need a sort]
 //   -> exclusive scan of kept counts -> compact -> (window, dim) counts -> scan = seg
 //   -> stable radix sort of kept entries by dim (input is in document order, so
 //      equal dims stay in ascending document id: the order is (dim, doc))
@@ -37,43 +37,236 @@ void launch_validate_indptr(const int64_t* indptr, int64_t n, uint32_t* err, cud
     SINDI_CUDA(cudaGetLastError());
 }
 
-// One warp per document. Validates the row (dims in range, finite values, no
-// duplicate dim), computes r_i = |alpha-mass(x_i)| (or, when vn > 0, r_i =
-// min(vn, nnz): Vector Number Pruning) and writes the kept entries (in pi
-// order) to kdim/kval at the row's own input positions.
-__global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(
-    const int64_t* indptr, const int32_t* indices, const float* values, int64_t n, int32_t dim, double alpha,
-    uint32_t vn, uint32_t* kept, int32_t* kdim, float* kval, uint32_t* long_rows, uint32_t* n_long, uint32_t* err) {
+// The kept set of a row is a bit mask: entry t of row i (indptr b) is bit t & 31 of word keep_words(b, i) + t / 32.
+// A row's words follow those of the row before it (ceil(m / 32) <= floor((b + m) / 32) - floor(b / 32) + 1), so the
+// whole mask takes nnz / 32 + n words: 1/64 of the kept entries' worst case.
+__host__ __device__ __forceinline__ int64_t keep_words(int64_t b, int64_t i) { return (b >> 5) + i; }
+
+struct PruneArgs {
+    const int64_t* indptr;
+    const int32_t* indices;
+    const float* values;
+    int64_t n;
+    int32_t dim;
+    double alpha;
+    uint32_t vn;           // > 0: Vector Number Pruning
+    uint32_t* kept;        // [n]
+    uint32_t* mask;        // kept set, see keep_words
+    uint32_t* sort_rows;   // rows left to prune_rows_kernel, and their count
+    uint32_t* n_sort;
+    uint32_t* long_rows;   // rows left to prune_long_rows_kernel, and their count
+    uint32_t* n_long;
+    uint32_t* err;
+};
+
+// ---------------------------------------------------------------------------
+// Pruning without a sort: one warp per row of up to 32 * I entries, I entries
+// per lane in registers. The kept set is a prefix of the pi order (|x|
+// descending, equal |x| by lower dim), so only its last |x|, K, is needed:
+// the largest K whose entries of |x| >= K reach alpha * mass (or vn entries).
+// K is found by bisecting the bit patterns of |x|, both ends pulled to the
+// nearest |x| of the row after every step (7 to 9 steps for 128 entries).
+//
+// The rule sums FP64 values one after another in pi order. The values are
+// FP32, so unless their magnitudes spread over 2^20 or more, every such sum
+// is exact and does not depend on the order: with all |x| whole multiples of
+// 2^low and their sum below 2^(low + 53), the sums are taken here as 64-bit
+// integers in units of 2^low, and the kept count is bit-identical. Rows for
+// which this does not hold, rows whose dims do not ascend (their duplicates
+// need a sort to be found) and rows of more than 512 entries go to
+// prune_rows_kernel.
+//
+// What bounds it: issue. A row of 120 entries takes about 450 warp
+// instructions, most of them in the bisection; a sorted row takes about 28
+// compare-exchange passes over shared memory and 2 * nnz dependent FP64 adds
+// by one lane (20.1 ms for 1M documents of 120 entries, alpha 0.5). Building
+// that index: 26.5 -> 7.4 ms.
+// ---------------------------------------------------------------------------
+constexpr int kSelectWarps = 8;
+constexpr int kSelectRowCap = 512;
+
+// Sum over the warp of one 53-bit share per lane (the total below 2^53): two 32-bit reductions.
+__device__ __forceinline__ uint64_t warp_sum53(uint64_t v) {
+    const uint32_t lo = __reduce_add_sync(kFull, (uint32_t)v & 0x3FFFFFFu);
+    const uint32_t hi = __reduce_add_sync(kFull, (uint32_t)(v >> 26));
+    return ((uint64_t)hi << 26) + lo;
+}
+
+// One row b .. b + m - 1 of at most 32 * I entries. False: the row is not for this path.
+template <int I>
+__device__ __forceinline__ bool prune_row_select(const PruneArgs& p, int64_t i, int64_t b, int m, int lane) {
+    uint32_t a[I];  // bits of |x|; 0: an explicit zero (not an entry) or past the row
+    bool bad_dim = false, bad_value = false, ascending = true;
+#pragma unroll
+    for (int u = 0; u < I; u++) {
+        const int t = lane + 32 * u;
+        a[u] = 0;
+        if (t < m) {
+            const int32_t j = __ldg(p.indices + b + t);
+            const int32_t before = t > 0 ? __ldg(p.indices + b + t - 1) : -1;
+            a[u] = __float_as_uint(__ldg(p.values + b + t)) & 0x7FFFFFFFu;
+            bad_dim |= j < 0 || j >= p.dim;
+            bad_value |= a[u] >= 0x7F800000u;
+            ascending &= before < j;
+        }
+    }
+    if (__any_sync(kFull, bad_dim || bad_value)) {
+        if (bad_dim) atomicOr(p.err, kErrDocDim);
+        if (bad_value) atomicOr(p.err, kErrDocValue);
+        if (lane == 0) p.kept[i] = 0;
+        return true;
+    }
+    if (!__all_sync(kFull, ascending)) return false;
+    uint32_t nz_l = 0, top_l = 0, least_l = 0xFFFFFFFFu;
+    int low_l = 1 << 20;
+#pragma unroll
+    for (int u = 0; u < I; u++) {
+        if (a[u]) {
+            nz_l++;
+            top_l = max(top_l, a[u]);
+            least_l = min(least_l, a[u]);
+            const int E = max(1, (int)(a[u] >> 23));
+            const uint32_t mant = a[u] >= 0x800000u ? (a[u] & 0x7FFFFFu) | 0x800000u : a[u];
+            low_l = min(low_l, E + __ffs(mant) - 1);
+        }
+    }
+    const uint32_t nz = __reduce_add_sync(kFull, nz_l);
+    uint32_t K = 1, ties = 0xFFFFFFFFu;  // kept: |x| > K, and the first `ties` entries of |x| == K
+    const bool by_mass = p.vn == 0;
+    if (nz && (by_mass ? p.alpha < 1.0 : p.vn < nz)) {
+        const uint32_t top = __reduce_max_sync(kFull, top_l);
+        const int low = by_mass ? __reduce_min_sync(kFull, low_l) : 0;
+        // every |x| is a multiple of 2^low and below 2^(Etop + 24) (both offset by 150)
+        if (by_mass && max(1, (int)(top >> 23)) + 24 + (32 - __clz((int)(nz - 1) | 1)) - low > 53) return false;
+        // an entry's share: |x| in units of 2^low, or 1 when entries are counted
+        auto share = [&](uint32_t x) -> uint64_t {
+            if (!by_mass) return 1;
+            const int E = max(1, (int)(x >> 23));
+            const uint64_t mant = x >= 0x800000u ? (x & 0x7FFFFFu) | 0x800000u : x;
+            return E >= low ? mant << (E - low) : mant >> (low - E);
+        };
+        uint64_t f[I];
+        uint64_t mine = 0;
+#pragma unroll
+        for (int u = 0; u < I; u++) {
+            f[u] = a[u] ? share(a[u]) : 0;
+            mine += f[u];
+        }
+        uint64_t target = p.vn;
+        if (by_mass) {
+            const uint64_t mass = warp_sum53(mine);
+            target = (uint64_t)ceil(__dmul_rn(p.alpha, (double)mass));  // prefix >= alpha * mass, for whole prefixes
+            if (target == 0) target = 1;
+        }
+        // lo: the least |x| known to reach the target with everything above it; hi: K < hi
+        uint32_t lo = __reduce_min_sync(kFull, least_l), hi = top + 1;
+        while (lo + 1 < hi) {
+            const uint32_t mid = lo + (hi - lo) / 2;  // lo < mid < hi
+            uint64_t s = 0;
+            uint32_t up = 0xFFFFFFFFu, down = 0;  // the nearest |x| of the row at or above mid, and below it
+#pragma unroll
+            for (int u = 0; u < I; u++) {
+                const bool ge = a[u] >= mid;
+                s += ge ? f[u] : 0ull;
+                up = ge ? min(up, a[u]) : up;
+                down = ge ? down : max(down, a[u]);
+            }
+            if (warp_sum53(s) >= target) {
+                lo = __reduce_min_sync(kFull, up);
+            } else {
+                hi = __reduce_max_sync(kFull, down) + 1;
+            }
+        }
+        K = lo;
+        uint64_t above = 0;
+#pragma unroll
+        for (int u = 0; u < I; u++) above += a[u] > K ? f[u] : 0ull;
+        above = warp_sum53(above);
+        const uint64_t fk = share(K);
+        // most rows: one entry of |x| == K, needed whole (target > above by the choice of K)
+        ties = target - above <= fk ? 1u : (uint32_t)((target - above + fk - 1) / fk);
+    }
+    uint32_t r = 0, tied = 0;
+    uint32_t* words = p.mask + keep_words(b, i);
+#pragma unroll
+    for (int u = 0; u < I; u++) {
+        if (32 * u < m) {
+            const unsigned eq = __ballot_sync(kFull, a[u] == K);
+            const bool keep = a[u] > K || (a[u] == K && tied + (uint32_t)__popc(eq & ((1u << lane) - 1u)) < ties);
+            tied += (uint32_t)__popc(eq);
+            const unsigned kw = __ballot_sync(kFull, keep);
+            r += (uint32_t)__popc(kw);
+            if (lane == 0) words[u] = kw;
+        }
+    }
+    if (lane == 0) p.kept[i] = r;
+    return true;
+}
+
+__global__ void __launch_bounds__(kSelectWarps * 32) prune_select_kernel(PruneArgs p) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = (int64_t)blockIdx.x * kSelectWarps + (threadIdx.x >> 5);
+    if (i >= p.n) return;
+    const int64_t b = p.indptr[i];
+    const int64_t m = p.indptr[i + 1] - b;
+    bool done;
+    if (m <= 64) done = prune_row_select<2>(p, i, b, (int)m, lane);
+    else if (m <= 128) done = prune_row_select<4>(p, i, b, (int)m, lane);
+    else if (m <= 256) done = prune_row_select<8>(p, i, b, (int)m, lane);
+    else if (m <= kSelectRowCap) done = prune_row_select<16>(p, i, b, (int)m, lane);
+    else done = false;
+    if (done || lane != 0) return;
+    if (m > kMaxRowNnz) {
+        atomicOr(p.err, kErrDocTooLong);
+        p.kept[i] = 0;
+    } else if (m > kPruneRowCap) {
+        p.long_rows[atomicAdd(p.n_long, 1u)] = (uint32_t)i;
+    } else {
+        p.sort_rows[atomicAdd(p.n_sort, 1u)] = (uint32_t)i;
+    }
+}
+
+// The mask words of a row whose pi order is in s (kept: its first r entries).
+// The row's threads t0, t0 + stride, ... (whole warps) call it.
+__device__ __forceinline__ void write_row_mask(const PruneArgs& p, int64_t i, int64_t b, int m, const uint64_t* s, int r,
+                                               int t0, int stride) {
+    const uint64_t last = r > 0 ? s[r - 1] : 0;
+    uint32_t* words = p.mask + keep_words(b, i);
+    for (int t = t0; t - (t0 & 31) < m; t += stride) {
+        bool keep = false;
+        if (t < m && r > 0) {
+            const float v = p.values[b + t];
+            keep = v != 0.0f && mass_key(p.indices[b + t], v) <= last;
+        }
+        const unsigned kw = __ballot_sync(kFull, keep);
+        if ((t & 31) == 0) words[t >> 5] = kw;
+    }
+}
+
+// One warp per listed row (rows prune_select_kernel leaves, at most kPruneRowCap
+// entries). Validates the row (dims in range, finite values, no duplicate dim)
+// and computes r_i = |alpha-mass(x_i)| (or, when vn > 0, r_i = min(vn, nnz):
+// Vector Number Pruning) from the sorted row.
+__global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(PruneArgs p) {
     __shared__ uint64_t sm[kPruneWarps][kPruneRowCap];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint64_t* s = sm[warp];
-    for (int64_t i = (int64_t)blockIdx.x * kPruneWarps + warp; i < n; i += (int64_t)gridDim.x * kPruneWarps) {
-        const int64_t b = indptr[i];
-        const int64_t m = indptr[i + 1] - b;
-        if (m > kPruneRowCap) {
-            if (lane == 0) {
-                if (m > kMaxRowNnz) {
-                    atomicOr(err, kErrDocTooLong);
-                    kept[i] = 0;
-                } else {
-                    uint32_t slot = atomicAdd(n_long, 1u);
-                    long_rows[slot] = (uint32_t)i;
-                }
-            }
-            continue;
-        }
-        const int mm = (int)m;
+    const uint32_t n_rows = *p.n_sort;
+    for (uint32_t row = blockIdx.x * kPruneWarps + warp; row < n_rows; row += gridDim.x * kPruneWarps) {
+        const int64_t i = p.sort_rows[row];
+        const int64_t b = p.indptr[i];
+        const int mm = (int)(p.indptr[i + 1] - b);
         int p2 = 32;
         while (p2 < mm) p2 <<= 1;
         // 1) dims: range check, and duplicates unless the row is strictly ascending
         bool bad = false, ascending = true;
         for (int t = lane; t < p2; t += 32) {
             if (t < mm) {
-                int32_t j = indices[b + t];
-                float v = values[b + t];
-                if (j < 0 || j >= dim) { bad = true; atomicOr(err, kErrDocDim); }
-                if (!isfinite(v)) { bad = true; atomicOr(err, kErrDocValue); }
-                if (t + 1 < mm && indices[b + t + 1] <= j) ascending = false;
+                int32_t j = p.indices[b + t];
+                float v = p.values[b + t];
+                if (j < 0 || j >= p.dim) { bad = true; atomicOr(p.err, kErrDocDim); }
+                if (!isfinite(v)) { bad = true; atomicOr(p.err, kErrDocValue); }
+                if (t + 1 < mm && p.indices[b + t + 1] <= j) ascending = false;
                 s[t] = ((uint64_t)(uint32_t)j << 32) | (uint32_t)t;
             } else {
                 s[t] = ~0ull;
@@ -83,7 +276,7 @@ __global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(
         ascending = __all_sync(kFull, ascending);
         __syncwarp();
         if (bad) {
-            if (lane == 0) kept[i] = 0;
+            if (lane == 0) p.kept[i] = 0;
             continue;
         }
         if (!ascending) {
@@ -95,8 +288,8 @@ __global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(
             __syncwarp();
             if (dup) {
                 if (lane == 0) {
-                    atomicOr(err, kErrDocDup);
-                    kept[i] = 0;
+                    atomicOr(p.err, kErrDocDup);
+                    p.kept[i] = 0;
                 }
                 continue;
             }
@@ -106,9 +299,9 @@ __global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(
         for (int t = lane; t < p2; t += 32) {
             uint64_t key = ~0ull;
             if (t < mm) {
-                float v = values[b + t];
+                float v = p.values[b + t];
                 if (v != 0.0f) {
-                    key = mass_key(indices[b + t], v);
+                    key = mass_key(p.indices[b + t], v);
                     nz++;
                 }
             }
@@ -119,101 +312,101 @@ __global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(
         __syncwarp();
         warp_bitonic_sort_asc(s, p2);
         int r = 0;
-        if (lane == 0) r = vn ? (nz < (int)vn ? nz : (int)vn) : alpha_mass_count(s, nz, alpha);
+        if (lane == 0) r = p.vn ? (nz < (int)p.vn ? nz : (int)p.vn) : alpha_mass_count(s, nz, p.alpha);
         r = __shfl_sync(kFull, r, 0);
-        for (int t = lane; t < r; t += 32) {
-            kdim[b + t] = mass_key_dim(s[t]);
-            kval[b + t] = mass_key_value(s[t]);
-        }
-        if (lane == 0) kept[i] = (uint32_t)r;
+        write_row_mask(p, i, b, mm, s, r, lane, 32);
+        if (lane == 0) p.kept[i] = (uint32_t)r;
         __syncwarp();
     }
 }
 
-// One block per long row (kPruneRowCap < m <= kMaxRowNnz); same rules.
+// One block per listed long row (kPruneRowCap < m <= kMaxRowNnz); same rules.
 constexpr int kLongBlock = 512;
-__global__ void __launch_bounds__(kLongBlock) prune_long_rows_kernel(
-    const int64_t* indptr, const int32_t* indices, const float* values, const uint32_t* rows, int32_t dim,
-    double alpha, uint32_t vn, uint32_t* kept, int32_t* kdim, float* kval, uint32_t* err) {
+__global__ void __launch_bounds__(kLongBlock) prune_long_rows_kernel(PruneArgs p) {
     extern __shared__ uint64_t s[];
     __shared__ int flags[2];
-    __shared__ int s_r;
-    const int64_t i = rows[blockIdx.x];
-    const int64_t b = indptr[i];
-    const int mm = (int)(indptr[i + 1] - b);
-    int p2 = 32;
-    while (p2 < mm) p2 <<= 1;
-    if (threadIdx.x == 0) { flags[0] = 0; flags[1] = 0; }
-    __syncthreads();
-    for (int t = threadIdx.x; t < p2; t += kLongBlock) {
-        if (t < mm) {
-            int32_t j = indices[b + t];
-            float v = values[b + t];
-            if (j < 0 || j >= dim) { flags[0] = 1; atomicOr(err, kErrDocDim); }
-            if (!isfinite(v)) { flags[0] = 1; atomicOr(err, kErrDocValue); }
-            s[t] = ((uint64_t)(uint32_t)j << 32) | (uint32_t)t;
-        } else {
-            s[t] = ~0ull;
-        }
-    }
-    __syncthreads();
-    if (flags[0]) {
-        if (threadIdx.x == 0) kept[i] = 0;
-        return;
-    }
-    // ascending sort of dims: reuse the descending sort on inverted keys
-    for (int t = threadIdx.x; t < p2; t += kLongBlock) s[t] = ~s[t];
-    __syncthreads();
-    block_bitonic_sort_desc<kLongBlock>(s, p2);
-    for (int t = threadIdx.x + 1; t < mm; t += kLongBlock)
-        if (((~s[t]) >> 32) == ((~s[t - 1]) >> 32)) flags[1] = 1;
-    __syncthreads();
-    if (flags[1]) {
-        if (threadIdx.x == 0) {
-            atomicOr(err, kErrDocDup);
-            kept[i] = 0;
-        }
-        return;
-    }
-    __shared__ int s_nz;
-    if (threadIdx.x == 0) s_nz = 0;
-    __syncthreads();
-    for (int t = threadIdx.x; t < p2; t += kLongBlock) {
-        uint64_t key = ~0ull;
-        if (t < mm) {
-            float v = values[b + t];
-            if (v != 0.0f) {
-                key = mass_key(indices[b + t], v);
-                atomicAdd(&s_nz, 1);
+    __shared__ int s_r, s_nz;
+    const uint32_t n_rows = *p.n_long;
+    for (uint32_t row = blockIdx.x; row < n_rows; row += gridDim.x) {
+        const int64_t i = p.long_rows[row];
+        const int64_t b = p.indptr[i];
+        const int mm = (int)(p.indptr[i + 1] - b);
+        int p2 = 32;
+        while (p2 < mm) p2 <<= 1;
+        __syncthreads();  // the previous row is done with the shared arrays
+        if (threadIdx.x == 0) { flags[0] = 0; flags[1] = 0; s_nz = 0; }
+        __syncthreads();
+        for (int t = threadIdx.x; t < p2; t += kLongBlock) {
+            if (t < mm) {
+                int32_t j = p.indices[b + t];
+                float v = p.values[b + t];
+                if (j < 0 || j >= p.dim) { flags[0] = 1; atomicOr(p.err, kErrDocDim); }
+                if (!isfinite(v)) { flags[0] = 1; atomicOr(p.err, kErrDocValue); }
+                s[t] = ((uint64_t)(uint32_t)j << 32) | (uint32_t)t;
+            } else {
+                s[t] = ~0ull;
             }
         }
-        s[t] = ~key;  // descending sort of inverted keys = ascending mass_key
+        __syncthreads();
+        if (flags[0]) {
+            if (threadIdx.x == 0) p.kept[i] = 0;
+            continue;
+        }
+        // ascending sort of dims: reuse the descending sort on inverted keys
+        for (int t = threadIdx.x; t < p2; t += kLongBlock) s[t] = ~s[t];
+        __syncthreads();
+        block_bitonic_sort_desc<kLongBlock>(s, p2);
+        for (int t = threadIdx.x + 1; t < mm; t += kLongBlock)
+            if (((~s[t]) >> 32) == ((~s[t - 1]) >> 32)) flags[1] = 1;
+        __syncthreads();
+        if (flags[1]) {
+            if (threadIdx.x == 0) {
+                atomicOr(p.err, kErrDocDup);
+                p.kept[i] = 0;
+            }
+            continue;
+        }
+        for (int t = threadIdx.x; t < p2; t += kLongBlock) {
+            uint64_t key = ~0ull;
+            if (t < mm) {
+                float v = p.values[b + t];
+                if (v != 0.0f) {
+                    key = mass_key(p.indices[b + t], v);
+                    atomicAdd(&s_nz, 1);
+                }
+            }
+            s[t] = ~key;  // descending sort of inverted keys = ascending mass_key
+        }
+        __syncthreads();
+        block_bitonic_sort_desc<kLongBlock>(s, p2);
+        for (int t = threadIdx.x; t < p2; t += kLongBlock) s[t] = ~s[t];
+        __syncthreads();
+        if (threadIdx.x == 0) s_r = p.vn ? (s_nz < (int)p.vn ? s_nz : (int)p.vn) : alpha_mass_count(s, s_nz, p.alpha);
+        __syncthreads();
+        const int r = s_r;
+        write_row_mask(p, i, b, mm, s, r, (int)threadIdx.x, kLongBlock);
+        if (threadIdx.x == 0) p.kept[i] = (uint32_t)r;
     }
-    __syncthreads();
-    block_bitonic_sort_desc<kLongBlock>(s, p2);
-    for (int t = threadIdx.x; t < p2; t += kLongBlock) s[t] = ~s[t];
-    __syncthreads();
-    if (threadIdx.x == 0) s_r = vn ? (s_nz < (int)vn ? s_nz : (int)vn) : alpha_mass_count(s, s_nz, alpha);
-    __syncthreads();
-    const int r = s_r;
-    for (int t = threadIdx.x; t < r; t += kLongBlock) {
-        kdim[b + t] = mass_key_dim(s[t]);
-        kval[b + t] = mass_key_value(s[t]);
-    }
-    if (threadIdx.x == 0) kept[i] = (uint32_t)r;
 }
 
-// Kept entries of every row -> compact arrays in document order.
-__global__ void compact_kernel(const int64_t* indptr, const int64_t* kept_off, const int32_t* kdim, const float* kval,
-                               int64_t n, uint32_t* sdim, uint32_t* sdoc, uint32_t* sval) {
+// Kept entries of every row -> compact arrays in document order (a warp per row).
+__global__ void compact_kernel(const int64_t* indptr, const int32_t* indices, const float* values, const uint32_t* mask,
+                               const int64_t* kept_off, int64_t n, uint32_t* sdim, uint32_t* sdoc, uint32_t* sval) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const int64_t b = indptr[i], o = kept_off[i], r = kept_off[i + 1] - o;
-        for (int64_t t = lane; t < r; t += 32) {
-            sdim[o + t] = (uint32_t)kdim[b + t];
-            sdoc[o + t] = (uint32_t)i;
-            sval[o + t] = __float_as_uint(kval[b + t]);
+        const int64_t b = indptr[i], m = indptr[i + 1] - b;
+        const uint32_t* words = mask + keep_words(b, i);
+        int64_t o = kept_off[i];
+        for (int64_t t0 = 0; t0 < m; t0 += 32) {
+            const uint32_t kw = words[t0 >> 5];
+            if ((kw >> lane) & 1u) {
+                const int64_t at = o + __popc(kw & ((1u << lane) - 1u));
+                sdim[at] = (uint32_t)indices[b + t0 + lane];
+                sdoc[at] = (uint32_t)i;
+                sval[at] = __float_as_uint(values[b + t0 + lane]);
+            }
+            o += __popc(kw);
         }
     }
 }
@@ -415,13 +608,6 @@ static uint32_t read_u32(const uint32_t* d, cudaStream_t s) {
     return h;
 }
 
-static int64_t read_i64(const int64_t* d, cudaStream_t s) {
-    int64_t h = 0;
-    SINDI_CUDA(cudaMemcpyAsync(&h, d, 8, cudaMemcpyDeviceToHost, s));
-    SINDI_CUDA(cudaStreamSynchronize(s));
-    return h;
-}
-
 static std::string doc_error_text(uint32_t e) {
     std::string m;
     if (e & kErrDocIndptr) m += "indptr[0] != 0 or decreasing; ";
@@ -453,41 +639,41 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
     ix.seg = P.alloc<uint32_t>((size_t)d * sigma + 1);
     const int64_t nnz = ix.doc_nnz;
     uint32_t* kept = ix.kept;
-    int32_t* kdim = P.alloc<int32_t>(nnz);
-    float* kval = P.alloc<float>(nnz);
-    uint32_t* long_rows = P.alloc<uint32_t>(n > 0 ? n : 1);
-    uint32_t* n_long = P.alloc<uint32_t>(1);
-    SINDI_CUDA(cudaMemsetAsync(n_long, 0, 4, stream));
-    SINDI_TRACE_MSG("build_lists: launching prune_rows");
+    const size_t mask_words = (size_t)keep_words(nnz, n) + 1;
+    uint32_t* mask = P.alloc<uint32_t>(mask_words);
+    uint32_t* left_rows = P.alloc<uint32_t>(2 * (size_t)n + 2);  // rows to sort, long rows, their counts
+    uint32_t* n_left = left_rows + 2 * n;
+    SINDI_CUDA(cudaMemsetAsync(n_left, 0, 8, stream));
+    SINDI_TRACE_MSG("build_lists: launching the pruning kernels");
+    int64_t* kept_off = P.alloc<int64_t>(n + 1);
     if (n > 0) {
-        prune_rows_kernel<<<grid_for(n, kPruneWarps, 152 * 32), kPruneWarps * 32, 0, stream>>>(
-            ix.indptr, ix.indices, ix.values, n, d, ix.alpha, vn, kept, kdim, kval, long_rows, n_long, ix.err);
+        const PruneArgs pa{ix.indptr, ix.indices, ix.values, n,         d,          ix.alpha,      vn,
+                           kept,      mask,       left_rows, n_left,    left_rows + n, n_left + 1, ix.err};
+        prune_select_kernel<<<(unsigned)((n + kSelectWarps - 1) / kSelectWarps), kSelectWarps * 32, 0, stream>>>(pa);
         SINDI_CUDA(cudaGetLastError());
-    }
-    uint32_t nl = n > 0 ? read_u32(n_long, stream) : 0;
-    if (nl > 0) {
-        size_t sm = (size_t)kMaxRowNnz * sizeof(uint64_t);
+        // the listed rows; their counts stay on the device
+        prune_rows_kernel<<<grid_for(n, kPruneWarps, 152 * 6), kPruneWarps * 32, 0, stream>>>(pa);
+        SINDI_CUDA(cudaGetLastError());
+        const size_t sm = (size_t)kMaxRowNnz * sizeof(uint64_t);
         SINDI_CUDA(cudaFuncSetAttribute(prune_long_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-        prune_long_rows_kernel<<<nl, kLongBlock, sm, stream>>>(ix.indptr, ix.indices, ix.values, long_rows, d,
-                                                                ix.alpha, vn, kept, kdim, kval, ix.err);
+        prune_long_rows_kernel<<<grid_for(n, 1, 152), kLongBlock, sm, stream>>>(pa);
         SINDI_CUDA(cudaGetLastError());
     }
+    exclusive_scan<uint32_t, int64_t>(kept, kept_off, n, P);
+    int64_t Pn0 = 0;
+    SINDI_CUDA(cudaMemcpyAsync(&Pn0, kept_off + n, 8, cudaMemcpyDeviceToHost, stream));
     e = read_u32(ix.err, stream);
+    P.free(left_rows);
     if (e) {
-        P.free(kdim); P.free(kval); P.free(long_rows); P.free(n_long);
+        P.free(mask); P.free(kept_off);
         set_last_error("malformed documents: " + doc_error_text(e));
         return (e & kErrDocTooLong) && !(e & ~kErrDocTooLong) ? SINDI_ERR_UNSUPPORTED : SINDI_ERR_INVALID_DATA;
     }
-    P.free(long_rows);
-    P.free(n_long);
 
     SINDI_TRACE_MSG("build_lists: pruning done");
     // --- compact kept entries (document order)
-    int64_t* kept_off = P.alloc<int64_t>(n + 1);
-    exclusive_scan<uint32_t, int64_t>(kept, kept_off, n, P);
-    const int64_t Pn0 = read_i64(kept_off + n, stream);
     if (Pn0 > kMaxPostings) {
-        P.free(kdim); P.free(kval); P.free(kept_off);
+        P.free(mask); P.free(kept_off);
         set_last_error("more than 2^32 - 4096 kept entries");
         return SINDI_ERR_UNSUPPORTED;
     }
@@ -496,12 +682,11 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
     uint32_t* sdoc = P.alloc<uint32_t>(Pn);
     uint32_t* sval = P.alloc<uint32_t>(Pn);
     if (n > 0) {
-        compact_kernel<<<grid_for(n, 8, 152 * 32), 256, 0, stream>>>(ix.indptr, kept_off, kdim, kval, n, sdim, sdoc,
-                                                                     sval);
+        compact_kernel<<<grid_for(n, 8, 152 * 32), 256, 0, stream>>>(ix.indptr, ix.indices, ix.values, mask, kept_off, n,
+                                                                     sdim, sdoc, sval);
         SINDI_CUDA(cudaGetLastError());
     }
-    P.free(kdim);
-    P.free(kval);
+    P.free(mask);
     P.free(kept_off);
 
     SINDI_TRACE_MSG("build_lists: compacted %lld kept entries", (long long)Pn);
