@@ -36,6 +36,7 @@
 #include <mutex>
 #include <vector>
 
+#include "bound_bins.cuh"
 #include "common.cuh"
 #include "fixed_point.cuh"
 #include "index.cuh"
@@ -53,7 +54,7 @@ constexpr uint32_t kSplitFraction = 8;     // its first 1/kSplitFraction windows
 constexpr int kMaxScanWarps = 1024 / 32;   // largest scan block
 constexpr int kChunkTable = 2048;          // chunks mapped to their list by a table (then a search)
 constexpr int kHistBits = 12;
-constexpr int kHistBins = 1 << kHistBits;  // bins on the top 12 bits of a score key
+constexpr int kHistBins = 1 << kHistBits;  // a window cut's bins: the top 12 bits of a score key
 constexpr int kKeyBinShift = 64 - kHistBits;
 constexpr int kSubBits = 8;                // second-level bins inside the cut bin
 constexpr int kSubBins = 1 << kSubBits;
@@ -73,7 +74,8 @@ struct Workspace {
     uint32_t* mticket;      // merge: finished blocks
     uint32_t* rticket;      // rerank: finished blocks
     uint32_t* top_count;    // reorder candidates
-    uint32_t* hist;         // [kHistBins] histogram of emitted candidates
+    uint32_t* qtop;         // the top bin of H, see hbin_top
+    uint32_t* hist;         // [kHBins] histogram H of emitted candidates
     uint64_t* cand;         // [cand_cap]
     uint64_t* fbuf;         // [fcap]
     uint64_t* top;          // [top_cap]
@@ -83,7 +85,9 @@ struct Workspace {
 
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
-// Bytes of a workspace for c queries, counters first (one memset clears them).
+// Bytes of a workspace for c queries, counters first (one memset of workspace_clear_bytes clears them). The
+// counters' room is that of the largest layout they ever had, so that what fits a fixed scratch area stays as it is.
+static size_t workspace_clear_bytes(int64_t c) { return (size_t)c * 4 * (6 + kHBins); }
 static size_t workspace_counter_bytes(int64_t c) { return align256((size_t)c * 4 * (5 + kHistBins)); }
 static size_t workspace_bytes(int64_t c, uint32_t cand_cap, uint32_t fcap, uint32_t top_cap) {
     return workspace_counter_bytes(c) + align256((size_t)c * cand_cap * 8) + align256((size_t)c * fcap * 8) +
@@ -94,11 +98,12 @@ static Workspace carve_workspace(unsigned char* base, int64_t c, uint32_t cand_c
     Workspace w;
     uint32_t* u = reinterpret_cast<uint32_t*>(base);
     w.hist = u;  // first: every query's row starts 16-byte aligned
-    w.cand_count = u + c * kHistBins;
+    w.cand_count = u + c * kHBins;
     w.fcount = w.cand_count + c;
     w.mticket = w.cand_count + 2 * c;
     w.rticket = w.cand_count + 3 * c;
     w.top_count = w.cand_count + 4 * c;
+    w.qtop = w.cand_count + 5 * c;
     unsigned char* q = base + workspace_counter_bytes(c);
     w.cand = reinterpret_cast<uint64_t*>(q);
     q += align256((size_t)c * cand_cap * 8);
@@ -186,10 +191,11 @@ __device__ __forceinline__ void load_ids8(const uint16_t* pid, uint32_t p0, uint
 template <int DT>
 __device__ __forceinline__ void load_values8(const void* pval, uint32_t p0, float v[8]) {
     if (DT == SINDI_F32) {
-        const float4* f = reinterpret_cast<const float4*>(static_cast<const float*>(pval) + p0);
-        const float4 a = __ldg(f), b = __ldg(f + 1);
-        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
-        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+        // one 32-byte load: the warp's 1 KiB is 8 lines; as two 16-byte loads a lane it is 16 half-used ones
+        // (the batched scan of the 1M-document workload, alone: 3.17 -> 3.06 ms)
+        asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                     : "l"(static_cast<const float*>(pval) + p0));
     } else if (DT == SINDI_F16) {
         const uint4 u = __ldg(reinterpret_cast<const uint4*>(static_cast<const __half*>(pval) + p0));
         const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
@@ -231,7 +237,6 @@ struct Chunk {
     float v[kChunkU];
     uint32_t lm;
     float wq;
-    uint32_t vec;               // a long segment's chunk: every lane's 8 ids were loaded
 };
 
 // Loads the chunk at offset `off` (a multiple of kChunkLen) of the segment
@@ -248,10 +253,8 @@ __device__ __forceinline__ void load_segment_chunk(const DevIndex& ix, uint32_t 
 #pragma unroll
     for (int u = 0; u < kChunkU / 2; u++) k.id2[u] = 0;
     k.lm = 0;
-    k.vec = 0;
     if (!checked(segment_in_bounds(ps, pe, ix.pcap), ix.err)) return;
     if (pe - ps >= kVecMin) {
-        k.vec = 1;
         const uint32_t q0 = (ps & ~7u) + off + (uint32_t)lane * kChunkU;
         const uint32_t lo = ps > q0 ? ps - q0 : 0u;  // < 8: only the segment's first group
         const uint32_t hi = pe > q0 ? min(pe - q0, (uint32_t)kChunkU) : 0u;
@@ -260,12 +263,6 @@ __device__ __forceinline__ void load_segment_chunk(const DevIndex& ix, uint32_t 
         if (k.lm) {
             load_ids8(ix.pid, q0, k.id2);
             load_values8<DT>(ix.pval, q0, k.v);
-            if (k.lm != 0xFFu) {
-                // a group at the segment's start or end: the postings outside it weigh 0
-#pragma unroll
-                for (int u = 0; u < kChunkU; u++)
-                    if (!((k.lm >> u) & 1u)) k.v[u] = 0.0f;
-            }
         }
     } else {
         const uint32_t q0 = ps + (uint32_t)lane;
@@ -292,17 +289,6 @@ __device__ __forceinline__ void load_chunk(const DevIndex& ix, const uint32_t* t
     load_segment_chunk<DT>(ix, t_start[t], t_end[t], (c - c_pre[t]) * (uint32_t)kChunkLen, lane, k);
 }
 
-// The same from the term table's packed records: {start, end, first chunk,
-// weight bits} per term, one 16-byte shared load.
-template <int DT>
-__device__ __forceinline__ void load_chunk_rec(const DevIndex& ix, const uint4* rec, const uint32_t* c_pre,
-                                               const uint16_t* c_term, int nc, uint32_t c, int lane, Chunk& k) {
-    const int t = c < (uint32_t)kChunkTable ? (int)c_term[c] : term_of(c_pre, nc, c);
-    const uint4 r = rec[t];
-    k.wq = __uint_as_float(r.w);
-    load_segment_chunk<DT>(ix, r.x, r.y, (c - r.z) * (uint32_t)kChunkLen, lane, k);
-}
-
 __device__ __forceinline__ uint32_t chunk_slot(const Chunk& k, int u) {
     return (k.id2[u >> 1] >> (16 * (u & 1))) & 0xFFFFu;
 }
@@ -314,29 +300,6 @@ __device__ __forceinline__ void add_chunk(float* A, uint32_t lambda, uint32_t* e
     for (int u = 0; u < kChunkU; u++)
         if ((k.lm & (1u << u)) && checked(slot_in_bounds(chunk_slot(k, u), lambda), err))
             atomicAdd(&A[chunk_slot(k, u)], k.wq * k.v[u]);
-}
-
-// The same into a fixed-point window: each product (its weight already
-// carries the window's 2^e) rounded to the nearest unit and added with a
-// native shared-memory integer atomic. In a long segment's chunk every lane
-// that loaded its group adds all 8 postings: the ones outside the segment
-// have value 0 (load_segment_chunk) and add 0 at the slot their load
-// returned (an id of a neighbouring segment, or the zero padding: a valid
-// slot, and an integer + 0 changes nothing), so the adds need no branch and
-// no select.
-__device__ __forceinline__ void add_chunk_fixed(int32_t* A, uint32_t lambda, uint32_t* err, const Chunk& k) {
-    if (k.vec && !kChecks) {
-        if (k.lm) {
-#pragma unroll
-            for (int u = 0; u < kChunkU; u++)
-                atomicAdd(&A[chunk_slot(k, u)], __float2int_rn(k.wq * k.v[u]));
-        }
-        return;
-    }
-#pragma unroll
-    for (int u = 0; u < kChunkU; u++)
-        if ((k.lm & (1u << u)) && checked(slot_in_bounds(chunk_slot(k, u), lambda), err))
-            atomicAdd(&A[chunk_slot(k, u)], __float2int_rn(k.wq * k.v[u]));
 }
 
 // Chunks of a segment of at least kVecMin postings.
@@ -390,14 +353,49 @@ __device__ void block_find_bin(const Get& get, uint32_t g, uint32_t* red, uint32
     group_find_bin<BINS, SyncBlock<BLOCK>>(get, g, red, st);
 }
 
-// 16-byte asynchronous copy global -> shared (through L2), and its completion.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((uint32_t)__cvta_generic_to_shared(smem)),
-                 "l"(gmem)
-                 : "memory");
+// One warp: whether H holds g candidates, and the bin of the g-th from the top. H may grow meanwhile: any
+// snapshot bounds the answer.
+__device__ __forceinline__ bool warp_find_bound(const uint32_t* H, uint32_t g, uint32_t* bin) {
+    constexpr int K = kHBins / 128;
+    const int lane = threadIdx.x & 31;
+    const uint4* H4 = reinterpret_cast<const uint4*>(H);
+    uint4 h[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) h[k] = __ldcg(H4 + (K - 1 - k) * 32 + lane);  // 128 bins a step, from the top
+    uint32_t above = 0, part = 0;
+    uint4 at = make_uint4(0, 0, 0, 0);
+    bool found = false;
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        const uint32_t tot = __reduce_add_sync(kFull, h[k].x + h[k].y + h[k].z + h[k].w);
+        if (!found) {
+            if (above + tot >= g) {
+                found = true;
+                at = h[k];
+                part = (uint32_t)(K - 1 - k);
+            } else {
+                above += tot;
+            }
+        }
+    }
+    if (!found) return false;
+    const uint32_t mine = at.x + at.y + at.z + at.w;
+    uint32_t incl = mine;  // this lane's and the higher lanes' bins
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_down_sync(kFull, incl, o);
+        if (lane + o < 32) incl += y;
+    }
+    uint32_t c = above + incl - mine;  // candidates above this lane's bins
+    const bool here = c < g && g <= c + mine;
+    uint32_t b = 128 * part + 4 * (uint32_t)lane;
+    if (g <= c + at.w) b += 3;
+    else if (g <= c + at.w + at.z) b += 2;
+    else if (g <= c + at.w + at.z + at.y) b += 1;
+    const unsigned who = __ballot_sync(kFull, here);
+    *bin = __shfl_sync(kFull, b, __ffs(who) - 1);
+    return true;
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 struct ScanArgs {
     DevIndex ix;
@@ -407,10 +405,10 @@ struct ScanArgs {
     int64_t q_first;
     uint32_t g;             // candidates per query: min(gamma or k, N)
     uint32_t win_cap;       // most candidates one window may emit without an exact select
-    int use_partial;        // read the per-query histogram before emitting: 0 no; 1 copied at the
-                            // block's start (batched: earlier windows of the query are done); 2 read
-                            // after the accumulation, once the previous launch (the query's first
-                            // windows) is complete
+    int use_partial;        // read the per-query histogram before emitting: 0 no; 1 at the block's
+                            // start (batched: earlier windows of the query are done); 2 after the
+                            // accumulation, once the previous launch (the query's first windows) is
+                            // complete
     uint32_t w0;            // first window of this launch
     uint32_t nq;            // pipelined scan: query rows and windows of the launch's items
     uint32_t nwin;
@@ -420,7 +418,8 @@ struct ScanArgs {
 
 // Shared-memory scratch of one window cut, owned by the threads that select.
 struct CutScratch {
-    uint32_t* hist;         // [kHistBins]
+    uint32_t* hist;         // [kHistBins]; may be the start of the region
+    uint32_t* rel_hist;     // [kRelBins]
     uint32_t* hist2;        // [kSubBins]
     unsigned char* region;  // per-warp private histograms, then staged keys (16-byte aligned)
     uint32_t region_bytes;
@@ -437,131 +436,193 @@ struct CutScratch {
 // window.
 // ---------------------------------------------------------------------------
 
-// A warp's share of B and of max |w_j| (b, m: this thread's terms) into
-// fred[warp] and fred[nw + warp]; every lane of the warp calls it.
-__device__ __forceinline__ void fx_warp_partials(float b, float m, float* fred, int warp, int nw) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        b += __shfl_xor_sync(kFull, b, o);
-        m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        fred[warp] = b;
-        fred[nw + warp] = m;
-    }
-}
+// What the block-wide table of a (query, window) reduces over the query's terms, one entry per warp.
+template <int NW>
+struct TermRed {
+    float b[NW];         // fixed-point window: this warp's terms' part of B
+    uint32_t m[NW];      // and of max |w_j| (bits of a non-negative float)
+    uint32_t q[NW];      // and of the query's largest product bound max_j |w_j| vmax_j, any window
+    uint32_t groups[NW]; // posting groups of the warp's terms
+};
 
-// e from the nw warps' partials (after a barrier). The warps are summed in a
-// fixed order, so every thread gets the same e.
-__device__ __forceinline__ int fx_exponent(const float* fred, int nw) {
-    float B = 0.0f, M = 0.0f;
-    for (int i = 0; i < nw; i++) {
-        B += fred[i];
-        M = fmaxf(M, fred[nw + i]);
-    }
-    return fx_exponent_from(B, M);
-}
-
-// This thread's part of B for term j of weight qv over window w.
-template <int DT>
-__device__ __forceinline__ void fx_term_bound(const DevIndex& ix, int32_t j, float qv, uint32_t len, float& b,
-                                              float& m) {
-    if (len == 0) return;
-    const float wq = fabsf((DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv);
-    b += wq * ix.vmax[j];
-    m = fmaxf(m, wq);
-}
-
-// The term table of one query over one window, for terms c0 .. c0 + nc - 1
-// of the query (nc <= the group's thread count): every term's posting range
-// and weight, and the map from warp chunks to terms. Returns the number of
-// chunks. Every thread of the group S calls it.
-template <int DT, typename S>
-__device__ uint32_t build_term_table(const ScanArgs& a, uint32_t w, int64_t qb, int c0, int nc, uint32_t* t_start,
-                                     uint32_t* t_end, float* t_w, uint32_t* c_pre, uint16_t* c_term, uint32_t* red,
-                                     uint32_t* negflag = nullptr, float* fred = nullptr, uint4* rec = nullptr) {
+// The term table of one query over one window for the window scan, for terms c0 .. c0 + nc - 1 of the query (nc <=
+// BLOCK, one term a thread). A term's segment is tiled on 8-aligned groups of 8 postings; the groups of all terms,
+// in term order, are numbered through, and a warp chunk is 32 consecutive groups, one a lane, whatever terms they
+// belong to:
+//   rec[t] = {first posting of the term's first group - 8 * number of that group (mod 2^32), segment start,
+//             segment end, weight (times 2^e in a fixed-point window)}
+//   pre[t] = number of term t's first group, pre[nc] = all groups (returned)
+//   c_term[c] = the term of chunk c's first group (chunks below kChunkTable)
+// Lanes of a chunk that crosses terms step on from there. (With a chunk per term, the 120 uniform terms of an
+// exact search had 8 of 32 lanes busy, and every segment below 32 postings cost a chunk of its own.)
+// j, qv: this thread's query entry (loaded by the caller, before it zeroes the window). fx_e: the window's exponent,
+// from this table's terms unless `fx_known`; qmax: raised to the terms' largest product bound. Every thread of the
+// block calls it.
+template <int DT, int BLOCK, bool FX>
+__device__ __forceinline__ uint32_t build_group_table(const ScanArgs& a, uint32_t w, int32_t j, float qv, int nc,
+                                                      uint4* rec, uint32_t* pre, uint16_t* c_term,
+                                                      TermRed<BLOCK / 32>& red, uint32_t* negflag, bool fx_known,
+                                                      int& fx_e, uint32_t& qmax) {
     const DevIndex& ix = a.ix;
-    const int tid = S::tid();
-    uint32_t nch = 0;
-    float fb = 0.0f, fm = 0.0f;  // fixed-point window: this thread's part of B and of max |w_j|
-    uint32_t r_start = 0, r_end = 0;  // the term's packed record (rec), once its first chunk is known
-    float r_w = 0.0f;
-    if (tid < nc) {
-        const int32_t j = a.q_indices[qb + c0 + tid];
-        const float qv = a.q_values[qb + c0 + tid];
-        if (negflag && qv < 0.0f) *negflag = 1u;  // a negative query value (any thread may set it)
-        uint32_t start = 0, len = 0;
-        float wq = 0.0f;
-        if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
-            const uint64_t sg = (uint64_t)j * ix.sigma + w;
-            start = ix.seg[sg];
-            len = ix.seg[sg + 1] - start;
-            wq = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
-        } else if (w == 0) {
-            atomicOr(ix.err, (j < 0 || j >= ix.dim) ? kErrQueryDim : kErrQueryValue);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int nwt = (nc + 31) >> 5;  // warps with terms
+    uint32_t start = 0, len = 0, ng = 0, excl = 0;
+    float wq = 0.0f;
+    if (warp < nwt) {
+        float fb = 0.0f, fm = 0.0f, fq = 0.0f;
+        if (tid < nc) {
+            if (qv < 0.0f) *negflag = 1u;  // a negative query value (any thread may set it)
+            if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
+                const uint64_t sg = (uint64_t)j * ix.sigma + w;
+                start = ix.seg[sg];
+                len = ix.seg[sg + 1] - start;
+                const float vm = ix.vmax[j];
+                wq = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
+                fq = fmaxf(0.0f, fabsf(wq) * vm);
+                if (FX && len) {
+                    fb = fabsf(wq) * vm;
+                    fm = fabsf(wq);
+                }
+                if (!checked(segment_in_bounds(start, start + len, ix.pcap), ix.err)) len = 0;
+            } else if (w == 0) {
+                atomicOr(ix.err, (j < 0 || j >= ix.dim) ? kErrQueryDim : kErrQueryValue);
+            }
+            ng = len ? ((start + len + 7u) >> 3) - (start >> 3) : 0u;
         }
-        t_start[tid] = start;
-        t_end[tid] = start + len;
-        t_w[tid] = wq;
-        r_start = start;
-        r_end = start + len;
-        r_w = wq;
-        if (fred) fx_term_bound<DT>(ix, j, qv, len, fb, fm);
-        // chunks of a long list tile its 8-aligned groups of postings
-        nch = len >= kVecMin ? (((start + len + 7u) & ~7u) - (start & ~7u) + kChunkLen - 1) / kChunkLen
-                             : (len ? 1u : 0u);
+        uint32_t incl = ng;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t up = __shfl_up_sync(kFull, incl, o);
+            if (lane >= o) incl += up;
+        }
+        excl = incl - ng;
+        if (FX && !fx_known) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) fb += __shfl_xor_sync(kFull, fb, o);
+            const uint32_t m = __reduce_max_sync(kFull, __float_as_uint(fm));
+            if (lane == 0) {
+                red.b[warp] = fb;
+                red.m[warp] = m;
+            }
+        }
+        const uint32_t q = __reduce_max_sync(kFull, __float_as_uint(fq));
+        if (lane == 0) red.q[warp] = q;
+        if (lane == 31) red.groups[warp] = incl;
     }
-    // (fred's partials are visible after the sum's barriers)
-    if (fred) fx_warp_partials(fb, fm, fred, tid >> 5, S::kThreads / 32);
-    uint32_t total;
-    const uint32_t excl = group_exclusive_sum<uint32_t, S>(nch, &total, red);
+    __syncthreads();
+    uint32_t total = 0;
+    {
+        // the warps in a fixed order, so that every thread gets the same e
+        float B = 0.0f;
+        uint32_t M = 0;
+        for (int i = 0; i < nwt; i++) {
+            if (FX && !fx_known) {
+                B += red.b[i];
+                M = max(M, red.m[i]);
+            }
+            qmax = max(qmax, red.q[i]);
+            if (i == warp) excl += total;
+            total += red.groups[i];
+        }
+        if (FX && !fx_known) fx_e = fx_exponent_from(B, __uint_as_float(M));
+    }
     if (tid < nc) {
-        c_pre[tid] = excl;
-        if (rec) rec[tid] = make_uint4(r_start, r_end, excl, __float_as_uint(r_w));
-        for (uint32_t c = excl; c < excl + nch && c < (uint32_t)kChunkTable; c++) c_term[c] = (uint16_t)tid;
+        const float wr = FX ? wq * pow2f(fx_e) : wq;  // exact (the exponent's clamps)
+        rec[tid] = make_uint4((start & ~7u) - 8u * excl, start, start + len, __float_as_uint(wr));
+        pre[tid] = excl;
+        for (uint32_t c = (excl + 31u) >> 5; 32u * c < excl + ng && c < (uint32_t)kChunkTable; c++)
+            c_term[c] = (uint16_t)tid;
     }
-    S::sync();
+    if (tid == 0) pre[nc] = total;
+    __syncthreads();
     return total;
 }
 
-// Scatter-add of one term table into the window A (Alg. 2's product and
-// accumulation loops): warp `warp` of NW takes chunks warp, warp + NW, ...;
-// the next chunk's loads are issued before this chunk's adds.
-template <int DT, int NW, bool FIXED = false>
-__device__ __forceinline__ void accumulate_table(const DevIndex& ix, const uint32_t* t_start, const uint32_t* t_end,
-                                                 const float* t_w, const uint32_t* c_pre, const uint16_t* c_term,
-                                                 int nc, uint32_t total, int warp, int lane, float* A,
-                                                 float wscale = 1.0f, const uint4* rec = nullptr) {
-    // two chunks in registers, taking turns (no copy between them)
-    uint32_t c = (uint32_t)warp;
-    Chunk ka, kb;
-    auto load = [&](uint32_t cc, Chunk& k) {
-        if (rec) load_chunk_rec<DT>(ix, rec, c_pre, c_term, nc, cc, lane, k);
-        else load_chunk<DT>(ix, t_start, t_end, t_w, c_pre, c_term, nc, cc, lane, k);
-        if (FIXED) k.wq *= wscale;  // the fixed-point window's 2^e (exact)
-    };
-    auto add = [&](const Chunk& k) {
-        if (FIXED) add_chunk_fixed(reinterpret_cast<int32_t*>(A), ix.lambda, ix.err, k);
-        else add_chunk(A, ix.lambda, ix.err, k);
-    };
-    if (c < total) load(c, ka);
-    while (c < total) {
-        c += NW;
-        if (c < total) load(c, kb);
-        add(ka);
-        if (c >= total) break;
-        c += NW;
-        if (c < total) load(c, ka);
-        add(kb);
+// A lane's group of 8 postings in registers; bit u of lm is set for those inside the segment (0: no group).
+struct Group8 {
+    uint32_t id2[kChunkU / 2];  // window ids, two per word (low half first)
+    float v[kChunkU];
+    float w;
+    uint32_t lm;
+};
+
+// Loads chunk c of a group table: lane l takes group 32 c + l.
+template <int DT>
+__device__ __forceinline__ void load_group(const DevIndex& ix, const uint4* rec, const uint32_t* pre,
+                                           const uint16_t* c_term, int nc, uint32_t total, uint32_t c, int lane,
+                                           Group8& k) {
+    const uint32_t G = 32u * c + (uint32_t)lane;
+    k.lm = 0;
+    if (G < total) {
+        int t = c < (uint32_t)kChunkTable ? (int)c_term[c] : term_of(pre, nc, G);
+        while (pre[t + 1] <= G) t++;
+        const uint4 r = rec[t];
+        const uint32_t q0 = r.x + 8u * G;
+        k.w = __uint_as_float(r.w);
+        k.lm = 0xFFu;
+        if (checked(group_in_bounds(q0, ix.pcap), ix.err)) {
+            load_ids8(ix.pid, q0, k.id2);
+            load_values8<DT>(ix.pval, q0, k.v);
+            if (q0 < r.y || q0 + 8u > r.z) {
+                // a group at the segment's start or end: the postings outside it weigh 0
+                const uint32_t lo = r.y > q0 ? r.y - q0 : 0u, hi = min(r.z - q0, (uint32_t)kChunkU);
+                k.lm = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+#pragma unroll
+                for (int u = 0; u < kChunkU; u++)
+                    if (!((k.lm >> u) & 1u)) k.v[u] = 0.0f;
+            }
+        } else {
+            k.lm = 0;
+        }
     }
 }
 
-// The fixed-point window's e for a query of more terms than one term table
-// holds (its B must be known before the first table's adds): a pass over all
-// of them. Every thread of the block calls it; fred: [2 * BLOCK / 32] floats,
-// free on entry and on return.
+// Adds a lane's group to the window with shared-memory atomics (groups of different terms run at once and may
+// meet on a slot). Fixed point: each product (its weight carries the window's 2^e) is rounded to the nearest unit
+// and added with a native integer atomic; all 8 postings are added, those outside the segment as 0 at the slot
+// their load returned (an id of a neighbouring segment, or the zero padding: a valid slot, and an integer + 0
+// changes nothing), so the adds need no branch and no select.
+template <bool FX>
+__device__ __forceinline__ void add_group(float* A, uint32_t lambda, uint32_t* err, const Group8& k) {
+    if (k.lm == 0) return;
+#pragma unroll
+    for (int u = 0; u < kChunkU; u++) {
+        const uint32_t slot = (k.id2[u >> 1] >> (16 * (u & 1))) & 0xFFFFu;
+        if (FX && !kChecks) {
+            atomicAdd(reinterpret_cast<int32_t*>(A) + slot, __float2int_rn(k.w * k.v[u]));
+        } else if ((k.lm & (1u << u)) && checked(slot_in_bounds(slot, lambda), err)) {
+            if (FX) atomicAdd(reinterpret_cast<int32_t*>(A) + slot, __float2int_rn(k.w * k.v[u]));
+            else atomicAdd(A + slot, k.w * k.v[u]);
+        }
+    }
+}
+
+// Scatter-add of one group table into the window A (Alg. 2's product and accumulation loops): warp `warp` of NW
+// takes chunks warp, warp + NW, ...; two chunks sit in registers and take turns, the next one's loads issued
+// before this one's adds.
+template <int DT, int NW, bool FX>
+__device__ __forceinline__ void accumulate_groups(const DevIndex& ix, const uint4* rec, const uint32_t* pre,
+                                                  const uint16_t* c_term, int nc, uint32_t total, int warp, int lane,
+                                                  float* A) {
+    const uint32_t chunks = (total + 31u) >> 5;
+    uint32_t c = (uint32_t)warp;
+    Group8 ka, kb;
+    if (c < chunks) load_group<DT>(ix, rec, pre, c_term, nc, total, c, lane, ka);
+    while (c < chunks) {
+        c += NW;
+        if (c < chunks) load_group<DT>(ix, rec, pre, c_term, nc, total, c, lane, kb);
+        add_group<FX>(A, ix.lambda, ix.err, ka);
+        if (c >= chunks) break;
+        c += NW;
+        if (c < chunks) load_group<DT>(ix, rec, pre, c_term, nc, total, c, lane, ka);
+        add_group<FX>(A, ix.lambda, ix.err, kb);
+    }
+}
+
+// The fixed-point window's e for a query of more terms than one table holds (its B must be known before the first
+// table's adds): a pass over all of them. Every thread of the block calls it; red is free on entry and on return.
 template <int DT, int BLOCK>
-__device__ int window_scale_exp(const ScanArgs& a, uint32_t w, int64_t qb, int nt, float* fred) {
+__device__ int window_scale_exp(const ScanArgs& a, uint32_t w, int64_t qb, int nt, TermRed<BLOCK / 32>& red) {
     const DevIndex& ix = a.ix;
     float b = 0.0f, m = 0.0f;
     for (int t = threadIdx.x; t < nt; t += BLOCK) {
@@ -569,14 +630,97 @@ __device__ int window_scale_exp(const ScanArgs& a, uint32_t w, int64_t qb, int n
         const float qv = a.q_values[qb + t];
         if (j >= 0 && j < ix.dim && isfinite(qv) && list_in_bounds(j, w, ix.dim, ix.sigma)) {
             const uint64_t sg = (uint64_t)j * ix.sigma + w;
-            fx_term_bound<DT>(ix, j, qv, ix.seg[sg + 1] - ix.seg[sg], b, m);
+            if (ix.seg[sg + 1] != ix.seg[sg]) {
+                const float wq = fabsf((DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv);
+                b += wq * ix.vmax[j];
+                m = fmaxf(m, wq);
+            }
         }
     }
-    fx_warp_partials(b, m, fred, threadIdx.x >> 5, BLOCK / 32);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        b += __shfl_xor_sync(kFull, b, o);
+        m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red.b[threadIdx.x >> 5] = b;
+        red.m[threadIdx.x >> 5] = __float_as_uint(m);
+    }
     __syncthreads();
-    const int e = fx_exponent(fred, BLOCK / 32);
+    float B = 0.0f, M = 0.0f;
+    for (int i = 0; i < BLOCK / 32; i++) {
+        B += red.b[i];
+        M = fmaxf(M, __uint_as_float(red.m[i]));
+    }
+    const int e = fx_exponent_from(B, M);
     __syncthreads();
     return e;
+}
+
+// The term table of one query over one window for the pipelined scan, for terms c0 .. c0 + nc - 1 of the query (nc
+// <= the group's thread count): every term's posting range and weight, and the map from warp chunks (of one term
+// each) to terms. *qmax gets the terms' largest product bound (bits of a non-negative float). Returns the number of
+// chunks. Every thread of the group S calls it.
+template <int DT, typename S>
+__device__ uint32_t build_term_table(const ScanArgs& a, uint32_t w, int64_t qb, int c0, int nc, uint32_t* t_start,
+                                     uint32_t* t_end, float* t_w, uint32_t* c_pre, uint16_t* c_term, uint32_t* red,
+                                     uint32_t* qmax) {
+    const DevIndex& ix = a.ix;
+    const int tid = S::tid();
+    uint32_t nch = 0;
+    float fq = 0.0f;
+    if (tid == 0) *qmax = 0;
+    if (tid < nc) {
+        const int32_t j = a.q_indices[qb + c0 + tid];
+        const float qv = a.q_values[qb + c0 + tid];
+        uint32_t start = 0, len = 0;
+        float wq = 0.0f;
+        if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
+            const uint64_t sg = (uint64_t)j * ix.sigma + w;
+            start = ix.seg[sg];
+            len = ix.seg[sg + 1] - start;
+            wq = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
+            fq = fmaxf(0.0f, fabsf(wq) * ix.vmax[j]);
+        } else if (w == 0) {
+            atomicOr(ix.err, (j < 0 || j >= ix.dim) ? kErrQueryDim : kErrQueryValue);
+        }
+        t_start[tid] = start;
+        t_end[tid] = start + len;
+        t_w[tid] = wq;
+        // chunks of a long list tile its 8-aligned groups of postings
+        nch = len >= kVecMin ? long_segment_chunks(start, start + len) : (len ? 1u : 0u);
+    }
+    const uint32_t q = __reduce_max_sync(kFull, __float_as_uint(fq));
+    uint32_t total;
+    const uint32_t excl = group_exclusive_sum<uint32_t, S>(nch, &total, red);
+    if ((tid & 31) == 0) atomicMax(qmax, q);  // (zeroed before the sum's barriers)
+    if (tid < nc) {
+        c_pre[tid] = excl;
+        for (uint32_t c = excl; c < excl + nch && c < (uint32_t)kChunkTable; c++) c_term[c] = (uint16_t)tid;
+    }
+    S::sync();
+    return total;
+}
+
+// Scatter-add of one term table into the window A for the pipelined scan: warp `warp` of NW takes chunks warp,
+// warp + NW, ...; the next chunk's loads are issued before this chunk's adds.
+template <int DT, int NW>
+__device__ __forceinline__ void accumulate_table(const DevIndex& ix, const uint32_t* t_start, const uint32_t* t_end,
+                                                 const float* t_w, const uint32_t* c_pre, const uint16_t* c_term,
+                                                 int nc, uint32_t total, int warp, int lane, float* A) {
+    // two chunks in registers, taking turns (no copy between them)
+    uint32_t c = (uint32_t)warp;
+    Chunk ka, kb;
+    if (c < total) load_chunk<DT>(ix, t_start, t_end, t_w, c_pre, c_term, nc, c, lane, ka);
+    while (c < total) {
+        c += NW;
+        if (c < total) load_chunk<DT>(ix, t_start, t_end, t_w, c_pre, c_term, nc, c, lane, kb);
+        add_chunk(A, ix.lambda, ix.err, ka);
+        if (c >= total) break;
+        c += NW;
+        if (c < total) load_chunk<DT>(ix, t_start, t_end, t_w, c_pre, c_term, nc, c, lane, ka);
+        add_chunk(A, ix.lambda, ix.err, kb);
+    }
 }
 
 constexpr int kNoFx = 1 << 30;  // select_window: the window holds FP32 scores
@@ -604,14 +748,18 @@ __device__ __forceinline__ float key_floor_float(uint32_t k) {
     return order_bits_float(k);
 }
 
+constexpr uint32_t kOneWarpEmits = 512;  // staged keys of a bounded window that one warp writes out alone
+
 // The cut of one accumulated window w of query row y: emits into the query's
 // candidate list every slot that can still be among its best g, and adds what
 // it emitted to the query's histogram H (ids >= N are not candidates).
-// `bounded`: g candidates of the query already exist at or above bin pbin.
-// Every thread of the group S (NW warps) calls it; the workspace must be free.
-template <typename S, int NW, bool FX = false>
-__device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t y, bool bounded, uint32_t pbin,
-                              const CutScratch& cs, bool skip_zero = false, int fx_e = kNoFx) {
+// `bounded`: g candidates of the query already exist with order bits of at
+// least `bound`; top: H's top bin (hbin_top). Every thread of the group S (NW
+// warps) calls it; the workspace must be free, and *cs.s_staged 0. LAST: the
+// scratch is not used again (a bounded cut then ends without a barrier).
+template <typename S, int NW, bool FX = false, bool LAST = false>
+__device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t y, bool bounded, uint32_t bound,
+                              int32_t top, const CutScratch& cs, bool skip_zero = false, int fx_e = kNoFx) {
     constexpr int NT = S::kThreads;
     const DevIndex& ix = a.ix;
     const int tid = S::tid();
@@ -623,7 +771,7 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     uint32_t* st = cs.st;
     uint64_t* stage = reinterpret_cast<uint64_t*>(cs.region);
     const uint32_t stage_cap = cs.region_bytes / 8;
-    uint32_t* H = a.ws.hist + (size_t)y * kHistBins;
+    uint32_t* H = a.ws.hist + (size_t)y * kHBins;
     const uint32_t lambda = ix.lambda;
     const int64_t gbase = (int64_t)w * lambda;
     const int64_t rest = ix.n_docs - gbase;
@@ -639,104 +787,104 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         return result_key(fx ? (float)Ai[i] * fx_inv : A[i], (uint32_t)(gbase + i));
     };
     uint64_t* cand = a.ws.cand + (size_t)y * a.ws.cand_cap;
+    auto put = [&](uint32_t at, uint64_t key) {
+        if (at < a.ws.cand_cap) cand[at] = key;
+        else atomicOr(ix.err, kErrCandOverflow);
+    };
     if (bounded) {
-        // g candidates at or above bin pbin already exist, so only slots in
-        // bins >= pbin can be in the answer. With skip_zero (every score of
-        // the query is >= 0 and the earlier windows hold at least g slots, all
-        // with scores >= 0 and lower ids), a slot whose score is exactly 0 can
-        // never be either: when the bound reaches down to 0, only positive
-        // slots count. When the slots that can count fit the window's budget,
-        // emit all of them: no window histogram, no cut. One pass: every warp
-        // stages its slots in its own share of the staging area (in order, no
-        // atomics); then one reservation for the group.
-        const unsigned lt = (1u << lane) - 1u;
-        const uint32_t share = stage_cap / NW;
-        uint64_t* mine_st = stage + (size_t)warp * share;
-        // the window 4 slots per lane (one 16-byte load, one compare each against
-        // the least score that can count); the per-slot work runs only for the
-        // rare 128-slot spans that hold a candidate
-        float thr = key_floor_float(pbin << (32 - kHistBits));
+        // g candidates at or above the bound already exist, so only slots at or
+        // above it can be in the answer. With skip_zero (every score of the query
+        // is >= 0 and the earlier windows hold at least g slots, all with scores
+        // >= 0 and lower ids), a slot whose score is exactly 0 can never be
+        // either: when the bound reaches down to 0, only positive slots count.
+        // When the slots that can count fit the window's budget, emit all of
+        // them: no window histogram, no cut. One pass stages them (a shared
+        // counter: a few dozen a window), then one reservation for the group.
+        float thr = key_floor_float(bound);
         if (skip_zero && thr <= 0.0f) thr = __int_as_float(1);  // the least positive float (NaN stays NaN)
         const int n4 = (n_eff + 3) >> 2;
         const float4* A4 = reinterpret_cast<const float4*>(A);
         const int4* I4 = reinterpret_cast<const int4*>(A);
         const int32_t ithr = fx ? fx_threshold(thr, fx_e) : 0;
-        auto scan_bounded = [&](auto&& emit) -> uint32_t {
-            uint32_t cnt = 0;
-            for (int b4 = warp * 32; b4 < n4; b4 += NT) {
-                const int i4 = b4 + lane;
-                uint32_t m = 0;
-                if (i4 < n4) {
-                    if (fx) {
-                        const int4 x = I4[i4];
-                        m = (x.x >= ithr ? 1u : 0u) | (x.y >= ithr ? 2u : 0u) | (x.z >= ithr ? 4u : 0u) |
-                            (x.w >= ithr ? 8u : 0u);
-                    } else {
-                        const float4 x = A4[i4];
-                        m = (x.x >= thr ? 1u : 0u) | (x.y >= thr ? 2u : 0u) | (x.z >= thr ? 4u : 0u) |
-                            (x.w >= thr ? 8u : 0u);
+        // the window 4 slots per lane: one 16-byte load, a maximum and one compare; the per-slot work runs
+        // only for the rare lane that holds a candidate
+        auto scan_bounded = [&](auto&& emit) {
+            if (fx) {
+#pragma unroll 4
+                for (int i4 = tid; i4 < n4; i4 += NT) {
+                    const int4 x = I4[i4];
+                    if (max(max(x.x, x.y), max(x.z, x.w)) >= ithr) {
+                        const int i = 4 * i4;
+                        if (x.x >= ithr) emit(i);
+                        if (x.y >= ithr && i + 1 < n_eff) emit(i + 1);
+                        if (x.z >= ithr && i + 2 < n_eff) emit(i + 2);
+                        if (x.w >= ithr && i + 3 < n_eff) emit(i + 3);
                     }
-                    const int rem = n_eff - 4 * i4;
-                    if (rem < 4) m &= (1u << rem) - 1u;
-                }
-                if (!__any_sync(kFull, m != 0u)) continue;
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    const bool ok = (m >> c) & 1u;
-                    const unsigned bal = __ballot_sync(kFull, ok);
-                    if (ok) emit(4 * i4 + c, cnt + (uint32_t)__popc(bal & lt));
-                    cnt += (uint32_t)__popc(bal);
-                }
-            }
-            return cnt;
-        };
-        const uint32_t cnt = scan_bounded([&](int i, uint32_t at) {
-            if (at < share) mine_st[at] = key_of(i);
-        });
-        if (lane == 0) warp_off[warp] = cnt;
-        S::sync();
-        if (tid == 0) {
-            uint32_t acc = 0, over = 0;
-            for (int k = 0; k < NW; k++) {
-                const uint32_t c = warp_off[k];
-                over |= c > share ? 1u : 0u;
-                warp_off[k] = acc;
-                acc += c;
-            }
-            cs.s_staged[0] = acc;
-            st[1] = over;
-            st[0] = acc && acc <= a.win_cap ? atomicAdd(a.ws.cand_count + y, acc) : 0u;
-        }
-        S::sync();
-        const uint32_t n_hi = cs.s_staged[0];
-        if (n_hi <= a.win_cap) {
-            const uint32_t at0 = st[0] + warp_off[warp];
-            if (st[1] == 0) {
-                // the staged keys out, each counted in the query's histogram
-                for (uint32_t t = (uint32_t)lane; t < cnt; t += 32) {
-                    const uint64_t key = mine_st[t];
-                    if (at0 + t < a.ws.cand_cap) cand[at0 + t] = key;
-                    else atomicOr(ix.err, kErrCandOverflow);
-                    atomicAdd(H + (uint32_t)(key >> kKeyBinShift), 1u);
                 }
             } else {
-                // a warp had more slots than its share: read the window again
-                (void)scan_bounded([&](int i, uint32_t at) {
-                    const uint64_t key = key_of(i);
-                    if (at0 + at < a.ws.cand_cap) cand[at0 + at] = key;
-                    else atomicOr(ix.err, kErrCandOverflow);
-                    atomicAdd(H + (uint32_t)(key >> kKeyBinShift), 1u);
-                });
+#pragma unroll 4
+                for (int i4 = tid; i4 < n4; i4 += NT) {
+                    const float4 x = A4[i4];
+                    if (x.x >= thr || x.y >= thr || x.z >= thr || x.w >= thr) {
+                        const int i = 4 * i4;
+                        if (x.x >= thr) emit(i);
+                        if (x.y >= thr && i + 1 < n_eff) emit(i + 1);
+                        if (x.z >= thr && i + 2 < n_eff) emit(i + 2);
+                        if (x.w >= thr && i + 3 < n_eff) emit(i + 3);
+                    }
+                }
             }
-            S::sync();  // warp_off, st and the staging area are reused by the caller's next cut
+        };
+        scan_bounded([&](int i) {
+            const uint32_t at = atomicAdd(cs.s_staged, 1u);
+            if (at < stage_cap) stage[at] = key_of(i);
+        });
+        S::sync();
+        const uint32_t n = *cs.s_staged;
+        if (n <= a.win_cap) {
+            if (n <= kOneWarpEmits && n <= stage_cap) {
+                if (warp == 0 && n) {
+                    uint32_t base = 0;
+                    if (lane == 0) base = atomicAdd(a.ws.cand_count + y, n);
+                    base = __shfl_sync(kFull, base, 0);
+                    for (uint32_t t = (uint32_t)lane; t < n; t += 32) {
+                        const uint64_t key = stage[t];
+                        put(base + t, key);
+                        atomicAdd(H + hbin((uint32_t)(key >> 32), top), 1u);
+                    }
+                }
+            } else {
+                S::sync();  // everyone has read the counter
+                if (tid == 0) {
+                    st[0] = atomicAdd(a.ws.cand_count + y, n);
+                    *cs.s_staged = 0;
+                }
+                S::sync();
+                const uint32_t base = st[0];
+                if (n <= stage_cap) {
+                    for (uint32_t t = (uint32_t)tid; t < n; t += NT) {
+                        const uint64_t key = stage[t];
+                        put(base + t, key);
+                        atomicAdd(H + hbin((uint32_t)(key >> 32), top), 1u);
+                    }
+                } else {
+                    // more slots than the staging area holds: read the window again
+                    scan_bounded([&](int i) {
+                        const uint64_t key = key_of(i);
+                        put(base + atomicAdd(cs.s_staged, 1u), key);
+                        atomicAdd(H + hbin((uint32_t)(key >> 32), top), 1u);
+                    });
+                }
+            }
+            if (!LAST) S::sync();  // st, the counter and the staging area are reused by the caller's next cut
             return;
         }
         // too many: the cut below decides (group-uniform), on FP32 scores
         if (fx) {
             fx_window_to_float<S>(A, lambda, fx_e);
-            S::sync();
             fx = false;
         }
+        S::sync();
     }
     // level 1: 12-bit bins of the score key. Each warp counts its slots in a
     // private histogram of the 256 bins below the window's top bin (no
@@ -791,10 +939,10 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     for (int b = tid; b < kRelBins; b += NT) {
         uint32_t c = 0;
         for (int k = 0; k < NW; k++) c += reinterpret_cast<uint32_t*>(cs.region)[k * kRelBins + b];
-        hist[b] = c;  // hist[rel] = slots in bin top_bin - rel (rel 255: that bin and all below)
+        cs.rel_hist[b] = c;  // slots in bin top_bin - b (b 255: that bin and all below)
     }
     S::sync();
-    group_find_bin<kRelBins, S>([&](int b) { return hist[kRelBins - 1 - b]; }, g_w, red, st);
+    group_find_bin<kRelBins, S>([&](int b) { return cs.rel_hist[kRelBins - 1 - b]; }, g_w, red, st);
     const uint32_t rel_cut = kRelBins - 1 - st[0];
     uint32_t bw = top_bin - rel_cut;
     uint32_t above_bw = st[1];
@@ -817,16 +965,10 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         c_bw = st[1] + st[2];
         S::sync();
     }
-    // slots of the window in 12-bit bin b (b within the histogram kept above)
-    auto bin_count = [&](uint32_t b) -> uint32_t {
-        if (!relative) return hist[b];
-        const uint32_t rel = top_bin - b;
-        return rel < (uint32_t)kRelBins - 1 ? hist[rel] : 0u;
-    };
     wait_previous_kernels();  // the workspace is free from here on
     uint32_t lo = bw;
-    // g slots already emitted at or above a bin prove the answer lies there
-    if (bounded && pbin > lo) lo = pbin;
+    // g slots already emitted at or above the bound prove the answer lies there
+    if (bounded) lo = max(lo, bound >> (32 - kHistBits));
     const bool staged = relative && c_bw <= stage_cap;  // slots >= bin lo fit in the staging area
     uint32_t n_src = (uint32_t)n_eff;
     if (staged) {
@@ -896,6 +1038,7 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         // ties crowd the cut: exact best g_w of the window
         thr = group_select_threshold<S>(src_key, (int)n_src, (int)g_w, hist2, st);
     }
+    if (bounded) thr = max(thr, (uint64_t)bound << 32);
     // emit keys >= thr: count, reserve the group's range with one atomic, write
     uint32_t mine = 0;
     for (int i = tid; i < (int)n_src; i += NT)
@@ -905,63 +1048,54 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     if (tid == 0) st[0] = total ? atomicAdd(a.ws.cand_count + y, total) : 0u;
     S::sync();
     pos += st[0];
-    for (int i = tid; i < (int)n_src && mine; i += NT) {
-        const uint64_t key = src_key(i);
-        if (key >= thr) {
-            if (pos < a.ws.cand_cap) cand[pos] = key;
-            else atomicOr(ix.err, kErrCandOverflow);
-            pos++;
-            mine--;
-        }
+    for (int b0 = 0; b0 < (int)n_src; b0 += NT) {
+        const int i = b0 + tid;
+        const uint64_t key = i < (int)n_src ? src_key(i) : 0ull;
+        const bool out = i < (int)n_src && key >= thr;
+        if (out) put(pos++, key);
+        // into H, one add per bin and warp (ties may put a whole window into one bin)
+        const uint32_t bin = out ? hbin((uint32_t)(key >> 32), top) : (uint32_t)kHBins;
+        const unsigned peers = __match_any_sync(kFull, bin);
+        if (out && lane == __ffs(peers) - 1) atomicAdd(H + bin, (uint32_t)__popc(peers));
     }
-    // what was emitted, per 12-bit bin, into the query's histogram: every
-    // bin above the cut bin in full, the rest of the emitted slots in it
-    const uint32_t tb = (uint32_t)(thr >> kKeyBinShift);
-    uint32_t above_mine = 0;
-    for (int b = tid; b < kHistBins; b += NT) {
-        const uint32_t c = (uint32_t)b > tb ? bin_count((uint32_t)b) : 0u;
-        if (c) {
-            above_mine += c;
-            atomicAdd(H + b, c);
-        }
-    }
-    uint32_t above;
-    (void)group_exclusive_sum<uint32_t, S>(above_mine, &above, red);
-    if (tid == 0 && total > above) atomicAdd(H + tb, total - above);
     S::sync();  // hist, region and st are reused by the caller's next cut
 }
 
 // One block per (window, query): the term tables are staged in shared memory,
 // the block's warps scatter-add every term's postings of the window into A,
-// then the block cuts the window.
+// then the block cuts the window. Shared memory: the window's scores, and one
+// region that holds the term tables while postings are added and the cut's
+// histograms and staged candidates afterwards. The query's running bound is
+// found by one warp while the table's loads are in flight.
+// What bounds it: the SMs' issue slots and L1/shared data pipe (postings come
+// from L2). With chunks of one term each, a 12-bit H read by all threads and
+// a barrier per table step it took 126 instructions per 256 postings plus 14k
+// a block; 1,000 queries over 1M documents (16,384-slot windows): 3.59 ->
+// 2.74 ms a batch, over 8.8M (8,192 slots, FP16): 40.2 -> 27.8 ms, exact
+// search of uniform vectors (segments of 64 postings): 0.69 -> 0.40 ms.
 template <int DT, bool QUERY_MAJOR, int BLOCK, bool FX>
 __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanArgs a) {
-    constexpr int kScanThreads = BLOCK;
     constexpr int kScanWarps = BLOCK / 32;
     constexpr int kTermChunk = BLOCK;   // query terms staged per pass (one per thread)
     using S = SyncBlock<BLOCK>;
-    // Shared memory: the window's scores, two histograms, and one region that
-    // holds the term tables while postings are added and the staged
-    // candidates of the window afterwards.
-    constexpr int kTableBytes = 16 * kTermChunk + (((4 * kTermChunk + 1) * 4 + kChunkTable * 2 + 15) & ~15);
+    constexpr int kTableBytes = (16 * kTermChunk + (kTermChunk + 1) * 4 + kChunkTable * 2 + 15) & ~15;
     constexpr int kPrivBytes = kScanWarps * kRelBins * 4;
-    constexpr int kRegionBytes = kTableBytes > kPrivBytes ? kTableBytes : kPrivBytes;
+    constexpr int kCutBytes = kPrivBytes > kHistBins * 4 ? kPrivBytes : kHistBins * 4;
+    constexpr int kRegionBytes = kTableBytes > kCutBytes ? kTableBytes : kCutBytes;
     extern __shared__ float A[];                    // [lambda]
-    __shared__ uint32_t hist[kHistBins];
-    __shared__ uint32_t hist2[kSubBins];
     __shared__ __align__(16) unsigned char region[kRegionBytes];
+    __shared__ uint32_t rel_hist[kRelBins];
+    __shared__ uint32_t hist2[kSubBins];
     __shared__ uint32_t warp_off[kScanWarps];
     __shared__ uint32_t red[kScanWarps + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
-    __shared__ uint32_t s_qneg;  // the query has a negative value
-    __shared__ float fred[2 * kScanWarps];  // fixed-point window: the warps' parts of B and of max |w_j|
-    uint4* t_rec = reinterpret_cast<uint4*>(region);  // the terms' packed records, read once per chunk
-    uint32_t* t_start = reinterpret_cast<uint32_t*>(region + 16 * kTermChunk);
-    uint32_t* t_end = t_start + kTermChunk;
-    uint32_t* c_pre = t_end + kTermChunk;
-    float* t_w = reinterpret_cast<float*>(c_pre + kTermChunk + 1);
-    uint16_t* c_term = reinterpret_cast<uint16_t*>(t_w + kTermChunk);
+    __shared__ uint32_t s_qneg;      // the query has a negative value
+    __shared__ uint32_t s_bound[2];  // H holds g candidates; the g-th's bin
+    __shared__ TermRed<kScanWarps> tred;
+    uint4* t_rec = reinterpret_cast<uint4*>(region);
+    uint32_t* t_pre = reinterpret_cast<uint32_t*>(region + 16 * kTermChunk);
+    uint16_t* c_term = reinterpret_cast<uint16_t*>(t_pre + kTermChunk + 1);
 
     const DevIndex& ix = a.ix;
     const uint32_t w = a.w0 + (QUERY_MAJOR ? blockIdx.y : blockIdx.x);
@@ -969,44 +1103,55 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
     const int64_t r = a.q_first + y;
     const uint32_t lambda = ix.lambda;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t* H = a.ws.hist + (size_t)y * kHBins;
 
-    uint32_t* H = a.ws.hist + (size_t)y * kHistBins;
-    if (a.use_partial == 1) {
-        // the query's histogram of what its earlier windows emitted, copied
-        // while the window accumulates (a snapshot: H only grows during the
-        // launch, so any snapshot bounds the answer)
-        wait_previous_kernels();  // the workspace is free from here on
-        for (int c = threadIdx.x; c < kHistBins / 4; c += kScanThreads) cp_async16(hist + 4 * c, H + 4 * c);
-        cp_async_commit();
-    }
     const int64_t qb = a.q_indptr[r];
     const int nt = (int)(a.q_indptr[r + 1] - qb);
-    if (threadIdx.x == 0) s_qneg = 0;  // read after the term tables' barriers
-
-    {
-        float4* A4 = reinterpret_cast<float4*>(A);
-        for (uint32_t m = threadIdx.x; m < window_stride(lambda) / 4; m += kScanThreads)
-            A4[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x == 0) {  // read after the term tables' barriers
+        s_qneg = 0;
+        s_staged = 0;
+    }
+    // the window is zeroed in two halves, while the query's offsets and then its terms are on their way
+    float4* A4 = reinterpret_cast<float4*>(A);
+    const uint32_t n4 = window_stride(lambda) / 4, n4h = n4 / 2;
+    for (uint32_t m = threadIdx.x; m < n4h; m += BLOCK) A4[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+    int32_t j = -1;
+    float qv = 0.0f;
+    if ((int)threadIdx.x < nt) {
+        j = a.q_indices[qb + threadIdx.x];
+        qv = a.q_values[qb + threadIdx.x];
+    }
+    for (uint32_t m = n4h + threadIdx.x; m < n4; m += BLOCK) A4[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.use_partial == 1 && warp == kScanWarps - 1) {
+        // the histogram of what the query's earlier windows emitted (a snapshot:
+        // H only grows during the launch, so any snapshot bounds the answer)
+        wait_previous_kernels();  // the workspace is free from here on
+        uint32_t b = 0;
+        const bool f = warp_find_bound(H, a.g, &b);
+        if (lane == 0) {
+            s_bound[0] = f ? 1u : 0u;
+            s_bound[1] = b;
+        }
     }
 
     // fixed-point window: the unit 2^-e of this (query, window). B comes with the
     // term table when one table holds the query's terms, else from a pass of its own.
     int fx_e = 0;
+    uint32_t qmax = 0;  // the query's largest product bound (bits)
     const bool fx_pre = FX && nt > kTermChunk;
-    if (fx_pre) fx_e = window_scale_exp<DT, BLOCK>(a, w, qb, nt, fred);
-    for (int c0 = 0; c0 < nt; c0 += kTermChunk) {
+    if (fx_pre) fx_e = window_scale_exp<DT, BLOCK>(a, w, qb, nt, tred);
+    for (int c0 = 0; c0 == 0 || c0 < nt; c0 += kTermChunk) {
         const int nc = min(kTermChunk, nt - c0);
-        __syncthreads();  // previous chunk fully consumed
-        const uint32_t total = build_term_table<DT, S>(a, w, qb, c0, nc, t_start, t_end, t_w, c_pre, c_term, red,
-                                                       &s_qneg, FX && !fx_pre ? fred : nullptr, t_rec);
-        if (FX) {
-            if (!fx_pre) fx_e = fx_exponent(fred, kScanWarps);
-            accumulate_table<DT, kScanWarps, true>(ix, t_start, t_end, t_w, c_pre, c_term, nc, total, warp, lane, A,
-                                                   pow2f(fx_e), t_rec);
-        } else {
-            accumulate_table<DT, kScanWarps>(ix, t_start, t_end, t_w, c_pre, c_term, nc, total, warp, lane, A,
-                                             1.0f, t_rec);
+        if (c0) {
+            if ((int)threadIdx.x < nc) {
+                j = a.q_indices[qb + c0 + threadIdx.x];
+                qv = a.q_values[qb + c0 + threadIdx.x];
+            }
+            __syncthreads();  // previous table fully consumed
         }
+        const uint32_t total = build_group_table<DT, BLOCK, FX>(a, w, j, qv, nc, t_rec, t_pre, c_term, tred, &s_qneg,
+                                                                fx_pre, fx_e, qmax);
+        accumulate_groups<DT, kScanWarps, FX>(ix, t_rec, t_pre, c_term, nc, total, warp, lane, A);
     }
     __syncthreads();
 
@@ -1015,23 +1160,32 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
     // accumulation
     allow_next_kernel();
 
-    uint32_t pbin = 0;  // bin of the g-th emitted candidate, when g have been emitted
-    bool bounded = false;
-    if (a.use_partial == 1) {
-        cp_async_wait_all();
-        __syncthreads();
-        block_find_bin<kHistBins, kScanThreads>([&](int b) { return hist[b]; }, a.g, red, st);
-        bounded = st[3] >= a.g;
-        pbin = st[0];
-        __syncthreads();
-    } else if (a.use_partial == 2) {
-        wait_previous_kernels();  // the first windows' candidates are all in H
-        block_find_bin<kHistBins, kScanThreads>([&](int b) { return __ldcg(H + b); }, a.g, red, st);
-        bounded = st[3] >= a.g;
-        pbin = st[0];
-        __syncthreads();
+    const int32_t top = hbin_top(float_order_bits(__uint_as_float(qmax)));
+    if (w == 0 && threadIdx.x == 0) {
+        wait_previous_kernels();
+        a.ws.qtop[y] = (uint32_t)top;
     }
-    const CutScratch cs{hist, hist2, region, (uint32_t)kRegionBytes, warp_off, red, st, &s_staged};
+    bool bounded = false;
+    uint32_t bound = 0;  // order bits below which no slot can be in the answer, when g candidates exist
+    if (a.use_partial) {
+        if (a.use_partial == 2) {
+            if (warp == 0) {
+                wait_previous_kernels();  // the first windows' candidates are all in H
+                uint32_t b = 0;
+                const bool f = warp_find_bound(H, a.g, &b);
+                if (lane == 0) {
+                    s_bound[0] = f ? 1u : 0u;
+                    s_bound[1] = b;
+                }
+            }
+            __syncthreads();
+        }
+        bounded = s_bound[0] != 0;
+        bound = bounded ? hbin_floor(s_bound[1], top) : 0u;
+        wait_previous_kernels();
+    }
+    const CutScratch cs{reinterpret_cast<uint32_t*>(region), rel_hist, hist2, region, (uint32_t)kRegionBytes, warp_off,
+                        red, st, &s_staged};
     // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
     const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
     // a fixed-point window without a bound goes to FP32 for the full cut; a bounded one is read as integers
@@ -1039,7 +1193,8 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
         fx_window_to_float<S>(A, lambda, fx_e);
         S::sync();
     }
-    select_window<S, kScanWarps, FX>(a, A, w, y, bounded, pbin, cs, skip_zero, FX && bounded ? fx_e : kNoFx);
+    select_window<S, kScanWarps, FX, true>(a, A, w, y, bounded, bound, top, cs, skip_zero,
+                                           FX && bounded ? fx_e : kNoFx);
 }
 
 // ---------------------------------------------------------------------------
@@ -1079,12 +1234,14 @@ template <int DT>
 __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ uint32_t hist[kHistBins];
+    __shared__ uint32_t rel_hist[kRelBins];
     __shared__ uint32_t hist2[kSubBins];
     __shared__ uint32_t warp_off[kPipeCutWarps];
     __shared__ uint32_t red[kPipeCutWarps + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
     __shared__ uint32_t t_total[2];
+    __shared__ uint32_t t_qmax[2];
     __shared__ int t_nc[2];
     using S = SyncGroup<kBarCut, kPipeCutWarps * 32, kPipeAddWarps * 32>;
     const DevIndex& ix = a.ix;
@@ -1135,7 +1292,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
     }
 
     // ---- cut group: tables ahead, then the cut of every accumulated item
-    const CutScratch cs{hist, hist2, region, (uint32_t)kPipeRegionBytes, warp_off, red, st, &s_staged};
+    const CutScratch cs{hist, rel_hist, hist2, region, (uint32_t)kPipeRegionBytes, warp_off, red, st, &s_staged};
     uint32_t bi = 0;  // next stage to build: item bi, pass bp
     int bp = 0;
     auto build_next = [&](int t) {
@@ -1146,7 +1303,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
         const int c0 = bp * kPipeTerms;
         const int nc = nt - c0 < kPipeTerms ? (nt - c0 > 0 ? nt - c0 : 0) : kPipeTerms;
         const uint32_t total = build_term_table<DT, S>(a, w, qb, c0, nc, t_start(t), t_end(t), t_w(t), c_pre(t),
-                                                       c_term(t), red);
+                                                       c_term(t), red, &t_qmax[t]);
         if (S::tid() == 0) {
             t_total[t] = total;
             t_nc[t] = nc;
@@ -1170,9 +1327,12 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
         const uint32_t y = item_y(it), w = item_w(it);
         const int np = passes(y);
         const int b = it & 1;
+        uint32_t qmax = 0;
         for (int p = 0; p < np; p++, s++) {
             const int t = s & 1;
             named_sync(kBarFree + t);
+            qmax = max(qmax, t_qmax[t]);
+            S::sync();  // read before the table is built anew
             if (bi < n_my) {
                 build_next(t);
                 named_arrive(kBarReady + t);
@@ -1184,13 +1344,23 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
         if (it == 0) wait_previous_kernels();
         if (it + 1 == n_my) allow_next_kernel();
         // the query's running bound: g candidates emitted at or above a bin
-        const uint32_t* H = a.ws.hist + (size_t)y * kHistBins;
-        group_find_bin<kHistBins, S>([&](int bb) { return __ldcg(H + bb); }, a.g, red, st);
-        const bool bounded = st[3] >= a.g;
-        const uint32_t pbin = st[0];
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(qmax)));
+        if (S::tid() < 32) {
+            uint32_t hb = 0;
+            const bool f = warp_find_bound(a.ws.hist + (size_t)y * kHBins, a.g, &hb);
+            if (S::tid() == 0) {
+                st[0] = hb;
+                st[3] = f ? 1u : 0u;
+                s_staged = 0;
+                if (w == 0) a.ws.qtop[y] = (uint32_t)top;
+            }
+        }
+        S::sync();
+        const bool bounded = st[3] != 0;
+        const uint32_t bound = bounded ? hbin_floor(st[0], top) : 0u;
         S::sync();
         float* A = buf0 + (size_t)b * lam4;
-        select_window<S, kPipeCutWarps>(a, A, w, y, bounded, pbin, cs);
+        select_window<S, kPipeCutWarps>(a, A, w, y, bounded, bound, top, cs);
         for (uint32_t m = (uint32_t)S::tid(); m < lam4 / 4; m += S::kThreads)
             reinterpret_cast<float4*>(A)[m] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (it + 2 < n_my) named_arrive(kBarEmpty + b);
@@ -1271,6 +1441,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
     using S = SyncBlock<BLOCK>;
     extern __shared__ __align__(16) unsigned char gsm[];
     __shared__ uint32_t hist[kHistBins];
+    __shared__ uint32_t rel_hist[kRelBins];
     __shared__ uint32_t hist2[kSubBins];
     __shared__ uint32_t warp_off[NW];
     __shared__ uint32_t red[NW + 1];
@@ -1280,6 +1451,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
     __shared__ uint32_t mpre[kMaxGroup + 1];    // prefix of the members' term counts
     __shared__ int64_t mqb[kMaxGroup];          // first entry of each member's query row
     __shared__ uint32_t s_negmask;              // bit i: member i has a negative query value
+    __shared__ uint32_t s_qmax[kMaxGroup];      // the members' largest product bounds (bits)
     const ScanArgs& sa = a.s;
     const DevIndex& ix = sa.ix;
     const uint32_t lambda = ix.lambda;
@@ -1302,6 +1474,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
     float* t_w = reinterpret_cast<float*>(t_mask + kGroupEntries);
     uint16_t* c_term = reinterpret_cast<uint16_t*>(t_w + kGroupEntries * kMaxGroup);
 
+    if (tid < kMaxGroup) s_qmax[tid] = 0;
     if (tid < (int)qn) {
         const uint32_t y = first + (uint32_t)tid;
         const int64_t r = sa.q_first + y;
@@ -1353,6 +1526,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
                 my_slot = (int)s;
                 my_i = i;
                 my_w = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
+                atomicMax(&s_qmax[i], __float_as_uint(fmaxf(0.0f, fabsf(my_w) * ix.vmax[j])));
                 atomicOr(&hval[s], 1u << i);
             }
         }
@@ -1429,19 +1603,30 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
 
     allow_next_kernel();
     wait_previous_kernels();  // the workspace (candidates, H) is free from here on
-    const CutScratch cs{hist, hist2, region, (uint32_t)group_region_bytes(BLOCK), warp_off, red, st, &s_staged};
+    const CutScratch cs{hist, rel_hist, hist2, region, (uint32_t)group_region_bytes(BLOCK), warp_off, red, st,
+                        &s_staged};
     for (uint32_t i = 0; i < qn; i++) {
         const uint32_t y = mrow[i];
         // the query's running bound: g candidates emitted at or above some bin (H only
         // grows while the launch runs, so any read of it bounds the answer)
-        const uint32_t* H = sa.ws.hist + (size_t)y * kHistBins;
-        block_find_bin<kHistBins, BLOCK>([&](int b) { return __ldcg(H + b); }, sa.g, red, st);
-        const bool bounded = st[3] >= sa.g;
-        const uint32_t pbin = st[0];
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(s_qmax[i])));
+        if (warp == 0) {
+            uint32_t hb = 0;
+            const bool f = warp_find_bound(sa.ws.hist + (size_t)y * kHBins, sa.g, &hb);
+            if (lane == 0) {
+                st[0] = hb;
+                st[3] = f ? 1u : 0u;
+                s_staged = 0;
+                if (w == 0) sa.ws.qtop[y] = (uint32_t)top;
+            }
+        }
+        __syncthreads();
+        const bool bounded = st[3] != 0;
+        const uint32_t bound = bounded ? hbin_floor(st[0], top) : 0u;
         __syncthreads();
         // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
         const bool skip_zero = !((s_negmask >> i) & 1u) && ix.nonneg && (uint64_t)w * lambda >= sa.g;
-        select_window<S, NW>(sa, A + (size_t)i * lam4, w, y, bounded, pbin, cs, skip_zero);
+        select_window<S, NW>(sa, A + (size_t)i * lam4, w, y, bounded, bound, top, cs, skip_zero);
     }
 }
 
@@ -1583,7 +1768,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
     }
     wait_previous_kernels();
     const uint32_t C = min(ws.cand_count[y], ws.cand_cap);
-    uint32_t* H = ws.hist + (size_t)y * kHistBins;
+    uint32_t* H = ws.hist + (size_t)y * kHBins;
     // Every block takes one ticket on the query's way out, whatever path it takes; the last one leaves
     // the query's counters and H at zero for the next launch that uses this workspace. (A block must not
     // reset them while another block of the grid may still read H.)
@@ -1594,7 +1779,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
         __syncthreads();
         if (!s_last) return;
         __threadfence();
-        for (int b = threadIdx.x; b < kHistBins; b += kMergeThreads) H[b] = 0;
+        for (int b = threadIdx.x; b < kHBins; b += kMergeThreads) H[b] = 0;
         if (threadIdx.x == 0) {
             ws.cand_count[y] = 0;
             ws.fcount[y] = 0;
@@ -1610,9 +1795,9 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
     const uint64_t* cand = ws.cand + (size_t)y * ws.cand_cap;
 
     // bin of the g-th best candidate; every candidate below it is out
-    block_find_bin<kHistBins, kMergeThreads>([&](int b) { return __ldcg(H + b); }, g, red, st);
-    const uint32_t bstar = st[0];
-    const uint32_t S = st[1] + st[2];  // candidates in bins >= bstar
+    block_find_bin<kHBins, kMergeThreads>([&](int b) { return __ldcg(H + b); }, g, red, st);
+    const uint32_t floor_bits = hbin_floor(st[0], (int32_t)__ldcg(ws.qtop + y));
+    const uint32_t S = st[1] + st[2];  // candidates in that bin and above
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     uint64_t* dst = a.final_stage ? sel : ws.top + (size_t)y * ws.top_cap;
@@ -1634,7 +1819,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const uint32_t i = base + (uint32_t)(u * kMergeThreads) + threadIdx.x;
-                if (i < C && (uint32_t)(kk[u] >> kKeyBinShift) >= bstar &&
+                if (i < C && (uint32_t)(kk[u] >> 32) >= floor_bits &&
                     checked(doc_in_bounds(key_id(kk[u]), a.ix.n_docs), a.ix.err)) {
                     const uint32_t pos = atomicAdd(&s_n, 1u);
                     if (pos < ws.fcap) sbuf[pos] = kk[u];
@@ -1674,7 +1859,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
 #pragma unroll
             for (int u = 0; u < 4; u++) {
                 const uint32_t i = base + (uint32_t)(u * kMergeThreads) + threadIdx.x;
-                if (i < hi && (uint32_t)(kk[u] >> kKeyBinShift) >= bstar &&
+                if (i < hi && (uint32_t)(kk[u] >> 32) >= floor_bits &&
                     checked(doc_in_bounds(key_id(kk[u]), a.ix.n_docs), a.ix.err)) {
                     const uint32_t pos = atomicAdd(&s_n, 1u);
                     if (pos < ws.fcap) sbuf[pos] = kk[u];
@@ -1722,7 +1907,7 @@ __global__ void __launch_bounds__(kMergeThreads) merge_kernel(MergeArgs a) {
     }
     __syncthreads();
     // leave the query's counters at zero for the next launch
-    for (int b = threadIdx.x; b < kHistBins; b += kMergeThreads) H[b] = 0;
+    for (int b = threadIdx.x; b < kHBins; b += kMergeThreads) H[b] = 0;
     if (threadIdx.x == 0) {
         ws.cand_count[y] = 0;
         ws.fcount[y] = 0;
@@ -2299,7 +2484,7 @@ static void capture_plain_graph(const IndexImpl& ix, const Plan& pl, const Index
         SINDI_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
         capturing = true;
         for (int l = 0; l < lanes; l++)
-            SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_counter_bytes(1), cap));
+            SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_clear_bytes(1), cap));
         enqueue_plain_lanes(ix, pl, wss, q_indptr, q_indices, q_values, n_queries, k, out_ids, out_scores, cap, ls,
                             nullptr, evs, true);
         capturing = false;
@@ -2405,7 +2590,7 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
     std::vector<Workspace> wss;
     for (int l = 0; l < lanes; l++) {
         wss.push_back(carve_workspace(mem + ws_stride * l, chunk, pl.cand_cap, pl.fcap, pl.top_cap));
-        SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_counter_bytes(chunk), stream));
+        SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_clear_bytes(chunk), stream));
     }
     const Workspace& ws = wss[0];
     QueryCsr pruned{nullptr, nullptr, nullptr};
@@ -2557,7 +2742,7 @@ sindi_status search_noalloc_impl(const IndexImpl& ix, const int64_t* q_indptr, c
     }
     const Workspace ws = carve_workspace(base, chunk, pl.cand_cap, pl.fcap, pl.top_cap);
     // the array keeps the previous call's contents: clear the counters the kernels start from
-    SINDI_CUDA(cudaMemsetAsync(base, 0, workspace_counter_bytes(chunk), stream));
+    SINDI_CUDA(cudaMemsetAsync(base, 0, workspace_clear_bytes(chunk), stream));
     bool chained = false;
     for (int64_t q0 = 0; q0 < n_queries; q0 += chunk) {
         const uint32_t nq = (uint32_t)std::min<int64_t>(chunk, n_queries - q0);
@@ -2601,7 +2786,7 @@ sindi_status search_in_workspace(const IndexImpl& ix, const int64_t* q_indptr, c
     }
     unsigned char* base = static_cast<unsigned char*>(ws_base);
     const Workspace ws = carve_workspace(base, chunk, pl.cand_cap, pl.fcap, pl.top_cap);
-    SINDI_CUDA(cudaMemsetAsync(base, 0, workspace_counter_bytes(chunk), stream));
+    SINDI_CUDA(cudaMemsetAsync(base, 0, workspace_clear_bytes(chunk), stream));
     bool chained = false;
     for (int64_t q0 = 0; q0 < n_queries; q0 += chunk) {
         const uint32_t nq = (uint32_t)std::min<int64_t>(chunk, n_queries - q0);
