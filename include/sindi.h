@@ -155,8 +155,9 @@ typedef struct {
                               plans, servers and sindi_search_noalloc return
                               SINDI_ERR_UNSUPPORTED for beta < 1                    */
     uint32_t mode;         /* sindi_mode                                           */
-    uint32_t block_threads;/* window-scan shape: 0 = the default (one block of 512
-                              threads per window); 256, 512 or 1024 = one block
+    uint32_t block_threads;/* window-scan shape: 0 = the default (one block per
+                              window, its threads picked from the window's size
+                              and the launch); 256, 512 or 1024 = one block
                               of that many threads per window;
                               SINDI_SCAN_PIPELINED = one resident block per SM
                               that overlaps the scatter-add of one window with

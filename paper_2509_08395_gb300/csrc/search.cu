@@ -45,20 +45,19 @@
 
 namespace sindi {
 
-constexpr int kScanThreadsPlain = 512;     // two blocks per SM: the windows of concurrent queries interleave
-constexpr int kScanThreadsBatched = 512;   // many windows: two blocks per SM overlap their phases
 constexpr int kPlainLanes = 24;            // plain schedule: query chains in flight at once
 constexpr uint32_t kPlainPipeItems = 6;    // plain schedule, pipelined scan: windows per block
 constexpr uint32_t kSplitMinWindows = 8;   // plain schedule: a query of this many windows or more scans
 constexpr uint32_t kSplitFraction = 8;     // its first 1/kSplitFraction windows first
 constexpr int kMaxScanWarps = 1024 / 32;   // largest scan block
-constexpr int kChunkTable = 2048;          // chunks mapped to their list by a table (then a search)
-constexpr int kHistBits = 12;
-constexpr int kHistBins = 1 << kHistBits;  // a window cut's bins: the top 12 bits of a score key
+constexpr int kChunkTable = 1024;          // chunks mapped to their list by a table (then a search)
+constexpr int kHistBits = 12;              // a window cut's bins: the top 12 bits of a score key
 constexpr int kKeyBinShift = 64 - kHistBits;
 constexpr int kSubBits = 8;                // second-level bins inside the cut bin
 constexpr int kSubBins = 1 << kSubBits;
-constexpr int kRelBins = 256;              // window histogram bins below the window's top bin
+constexpr int kRelBins = 256;              // window histogram bins from the window's top bin down
+constexpr int kCutHists = 4;               // histograms the warps of a cut share
+static_assert(kRelBins <= kSubBins, "the window's histogram and the second level take turns in one array");
 constexpr int kMergeThreads = 512;
 constexpr uint32_t kMergeOneBlock = 16384;  // candidates one merge block gathers alone
 constexpr int kRerankThreads = 256;
@@ -88,7 +87,7 @@ static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 // Bytes of a workspace for c queries, counters first (one memset of workspace_clear_bytes clears them). The
 // counters' room is that of the largest layout they ever had, so that what fits a fixed scratch area stays as it is.
 static size_t workspace_clear_bytes(int64_t c) { return (size_t)c * 4 * (6 + kHBins); }
-static size_t workspace_counter_bytes(int64_t c) { return align256((size_t)c * 4 * (5 + kHistBins)); }
+static size_t workspace_counter_bytes(int64_t c) { return align256((size_t)c * 4 * (5 + 4096)); }
 static size_t workspace_bytes(int64_t c, uint32_t cand_cap, uint32_t fcap, uint32_t top_cap) {
     return workspace_counter_bytes(c) + align256((size_t)c * cand_cap * 8) + align256((size_t)c * fcap * 8) +
            2 * align256((size_t)c * top_cap * 8);
@@ -418,12 +417,9 @@ struct ScanArgs {
 
 // Shared-memory scratch of one window cut, owned by the threads that select.
 struct CutScratch {
-    uint32_t* hist;         // [kHistBins]; may be the start of the region
-    uint32_t* rel_hist;     // [kRelBins]
     uint32_t* hist2;        // [kSubBins]
-    unsigned char* region;  // per-warp private histograms, then staged keys (16-byte aligned)
+    unsigned char* region;  // the histograms of level 1, then staged keys (16-byte aligned)
     uint32_t region_bytes;
-    uint32_t* warp_off;     // [warps of the group]
     uint32_t* red;          // [warps of the group + 1]
     uint32_t* st;           // [4]
     uint32_t* s_staged;     // [1]
@@ -436,14 +432,22 @@ struct CutScratch {
 // window.
 // ---------------------------------------------------------------------------
 
-// What the block-wide table of a (query, window) reduces over the query's terms, one entry per warp.
+// What the block-wide table of a (query, window) reduces over the query's terms, one entry per warp, and its results.
 template <int NW>
 struct TermRed {
     float b[NW];         // fixed-point window: this warp's terms' part of B
     uint32_t m[NW];      // and of max |w_j| (bits of a non-negative float)
     uint32_t q[NW];      // and of the query's largest product bound max_j |w_j| vmax_j, any window
     uint32_t groups[NW]; // posting groups of the warp's terms
+    uint32_t total;      // posting groups of the table
+    uint32_t qmax;       // the query's largest product bound so far (0 before the first table)
+    int fx_e;            // fixed-point window: its exponent
 };
+
+// The block's barrier, for warps that reach it from different places.
+__device__ __forceinline__ void block_barrier() { asm volatile("barrier.cta.sync 0;" ::: "memory"); }
+
+constexpr uint32_t kPureChunk = 0x8000u;  // c_term: every group of the chunk is one term's, whole
 
 // The term table of one query over one window for the window scan, for terms c0 .. c0 + nc - 1 of the query (nc <=
 // BLOCK, one term a thread). A term's segment is tiled on 8-aligned groups of 8 postings; the groups of all terms,
@@ -451,94 +455,100 @@ struct TermRed {
 // belong to:
 //   rec[t] = {first posting of the term's first group - 8 * number of that group (mod 2^32), segment start,
 //             segment end, weight (times 2^e in a fixed-point window)}
-//   pre[t] = number of term t's first group, pre[nc] = all groups (returned)
-//   c_term[c] = the term of chunk c's first group (chunks below kChunkTable)
+//   pre[t] = number of term t's first group, pre[nc] = all groups (red.total)
+//   c_term[c] = the term of chunk c's first group (chunks below kChunkTable), with kPureChunk when the chunk needs
+//               no look at term or segment ends
 // Lanes of a chunk that crosses terms step on from there. (With a chunk per term, the 120 uniform terms of an
 // exact search had 8 of 32 lanes busy, and every segment below 32 postings cost a chunk of its own.)
-// j, qv: this thread's query entry (loaded by the caller, before it zeroes the window). fx_e: the window's exponent,
-// from this table's terms unless `fx_known`; qmax: raised to the terms' largest product bound. Every thread of the
-// block calls it.
+// j, qv: this thread's query entry (loaded by the caller, before it zeroes the window). red.fx_e comes from this
+// table's terms unless `fx_known`. Only the warps with terms compute; the others pass the two barriers. Every
+// thread of the block calls it.
 template <int DT, int BLOCK, bool FX>
-__device__ __forceinline__ uint32_t build_group_table(const ScanArgs& a, uint32_t w, int32_t j, float qv, int nc,
-                                                      uint4* rec, uint32_t* pre, uint16_t* c_term,
-                                                      TermRed<BLOCK / 32>& red, uint32_t* negflag, bool fx_known,
-                                                      int& fx_e, uint32_t& qmax) {
+__device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w, int32_t j, float qv, int nc, uint4* rec,
+                                                  uint32_t* pre, uint16_t* c_term, TermRed<BLOCK / 32>& red,
+                                                  uint32_t* negflag, bool fx_known) {
     const DevIndex& ix = a.ix;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nwt = (nc + 31) >> 5;  // warps with terms
-    uint32_t start = 0, len = 0, ng = 0, excl = 0;
-    float wq = 0.0f;
-    if (warp < nwt) {
-        float fb = 0.0f, fm = 0.0f, fq = 0.0f;
-        if (tid < nc) {
-            if (qv < 0.0f) *negflag = 1u;  // a negative query value (any thread may set it)
-            if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
-                const uint64_t sg = (uint64_t)j * ix.sigma + w;
-                start = ix.seg[sg];
-                len = ix.seg[sg + 1] - start;
-                const float vm = ix.vmax[j];
-                wq = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
-                fq = fmaxf(0.0f, fabsf(wq) * vm);
-                if (FX && len) {
-                    fb = fabsf(wq) * vm;
-                    fm = fabsf(wq);
-                }
-                if (!checked(segment_in_bounds(start, start + len, ix.pcap), ix.err)) len = 0;
-            } else if (w == 0) {
-                atomicOr(ix.err, (j < 0 || j >= ix.dim) ? kErrQueryDim : kErrQueryValue);
+    const int nwt = max(1, (nc + 31) >> 5);  // warps with terms
+    if (warp >= nwt) {
+        block_barrier();
+        block_barrier();
+        return;
+    }
+    uint32_t start = 0, len = 0;
+    float wq = 0.0f, fb = 0.0f, fm = 0.0f, fq = 0.0f;
+    if (tid < nc) {
+        if (qv < 0.0f) *negflag = 1u;  // a negative query value (any thread may set it)
+        if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
+            const uint64_t sg = (uint64_t)j * ix.sigma + w;
+            start = ix.seg[sg];
+            len = ix.seg[sg + 1] - start;
+            const float vm = ix.vmax[j];
+            wq = (DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv;
+            fq = fmaxf(0.0f, fabsf(wq) * vm);
+            if (FX && len) {
+                fb = fabsf(wq) * vm;
+                fm = fabsf(wq);
             }
-            ng = len ? ((start + len + 7u) >> 3) - (start >> 3) : 0u;
+            if (!checked(segment_in_bounds(start, start + len, ix.pcap), ix.err)) len = 0;
+        } else if (w == 0) {
+            atomicOr(ix.err, (j < 0 || j >= ix.dim) ? kErrQueryDim : kErrQueryValue);
         }
-        uint32_t incl = ng;
+    }
+    const uint32_t end = start + len;
+    const uint32_t ng = len ? ((end + 7u) >> 3) - (start >> 3) : 0u;
+    uint32_t incl = ng;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t up = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += up;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t up = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += up;
+    }
+    uint32_t excl = incl - ng;
+    if (FX && !fx_known) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fb += __shfl_xor_sync(kFull, fb, o);
+        const uint32_t m = __reduce_max_sync(kFull, __float_as_uint(fm));
+        if (lane == 0) {
+            red.b[warp] = fb;
+            red.m[warp] = m;
         }
-        excl = incl - ng;
+    }
+    const uint32_t q = __reduce_max_sync(kFull, __float_as_uint(fq));
+    if (lane == 0) red.q[warp] = q;
+    if (lane == 31) red.groups[warp] = incl;
+    block_barrier();
+    uint32_t total = 0, M = 0, Q = 0;
+    float B = 0.0f;
+    for (int i = 0; i < nwt; i++) {  // the warps in a fixed order, so that every thread gets the same e
         if (FX && !fx_known) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) fb += __shfl_xor_sync(kFull, fb, o);
-            const uint32_t m = __reduce_max_sync(kFull, __float_as_uint(fm));
-            if (lane == 0) {
-                red.b[warp] = fb;
-                red.m[warp] = m;
-            }
+            B += red.b[i];
+            M = max(M, red.m[i]);
         }
-        const uint32_t q = __reduce_max_sync(kFull, __float_as_uint(fq));
-        if (lane == 0) red.q[warp] = q;
-        if (lane == 31) red.groups[warp] = incl;
+        Q = max(Q, red.q[i]);
+        if (i == warp) excl += total;
+        total += red.groups[i];
     }
-    __syncthreads();
-    uint32_t total = 0;
-    {
-        // the warps in a fixed order, so that every thread gets the same e
-        float B = 0.0f;
-        uint32_t M = 0;
-        for (int i = 0; i < nwt; i++) {
-            if (FX && !fx_known) {
-                B += red.b[i];
-                M = max(M, red.m[i]);
-            }
-            qmax = max(qmax, red.q[i]);
-            if (i == warp) excl += total;
-            total += red.groups[i];
-        }
-        if (FX && !fx_known) fx_e = fx_exponent_from(B, __uint_as_float(M));
-    }
+    const int fx_e = FX ? (fx_known ? red.fx_e : fx_exponent_from(B, __uint_as_float(M))) : 0;
     if (tid < nc) {
         const float wr = FX ? wq * pow2f(fx_e) : wq;  // exact (the exponent's clamps)
-        rec[tid] = make_uint4((start & ~7u) - 8u * excl, start, start + len, __float_as_uint(wr));
+        rec[tid] = make_uint4((start & ~7u) - 8u * excl, start, end, __float_as_uint(wr));
         pre[tid] = excl;
+        const uint32_t whole0 = excl + ((start & 7u) ? 1u : 0u), whole1 = excl + ng - ((end & 7u) ? 1u : 0u);
         for (uint32_t c = (excl + 31u) >> 5; 32u * c < excl + ng && c < (uint32_t)kChunkTable; c++)
-            c_term[c] = (uint16_t)tid;
+            c_term[c] = (uint16_t)((uint32_t)tid |
+                                   (32u * c >= whole0 && 32u * c + 32u <= whole1 ? kPureChunk : 0u));
     }
-    if (tid == 0) pre[nc] = total;
-    __syncthreads();
-    return total;
+    if (tid == 0) {
+        pre[nc] = total;
+        red.total = total;
+        red.qmax = max(red.qmax, Q);
+        if (FX && !fx_known) red.fx_e = fx_e;
+    }
+    block_barrier();
 }
 
-// A lane's group of 8 postings in registers; bit u of lm is set for those inside the segment (0: no group).
+// A lane's group of 8 postings in registers. lm: bit u is set for a posting inside the segment (0: no group). The
+// others have value 0.
 struct Group8 {
     uint32_t id2[kChunkU / 2];  // window ids, two per word (low half first)
     float v[kChunkU];
@@ -552,39 +562,49 @@ __device__ __forceinline__ void load_group(const DevIndex& ix, const uint4* rec,
                                            const uint16_t* c_term, int nc, uint32_t total, uint32_t c, int lane,
                                            Group8& k) {
     const uint32_t G = 32u * c + (uint32_t)lane;
-    k.lm = 0;
-    if (G < total) {
-        int t = c < (uint32_t)kChunkTable ? (int)c_term[c] : term_of(pre, nc, G);
-        while (pre[t + 1] <= G) t++;
-        const uint4 r = rec[t];
+    const uint32_t ct = c < (uint32_t)kChunkTable ? (uint32_t)c_term[c] : (uint32_t)term_of(pre, nc, 32u * c);
+    k.lm = 0xFFu;
+    if (ct & kPureChunk) {
+        // about 7 in 10 chunks of the 1M-document workload
+        const uint4 r = rec[ct & ~kPureChunk];
         const uint32_t q0 = r.x + 8u * G;
         k.w = __uint_as_float(r.w);
-        k.lm = 0xFFu;
         if (checked(group_in_bounds(q0, ix.pcap), ix.err)) {
             load_ids8(ix.pid, q0, k.id2);
             load_values8<DT>(ix.pval, q0, k.v);
-            if (q0 < r.y || q0 + 8u > r.z) {
-                // a group at the segment's start or end: the postings outside it weigh 0
-                const uint32_t lo = r.y > q0 ? r.y - q0 : 0u, hi = min(r.z - q0, (uint32_t)kChunkU);
-                k.lm = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
-#pragma unroll
-                for (int u = 0; u < kChunkU; u++)
-                    if (!((k.lm >> u) & 1u)) k.v[u] = 0.0f;
-            }
-        } else {
-            k.lm = 0;
+            return;
         }
     }
+    k.w = 0.0f;
+    k.lm = 0;
+#pragma unroll
+    for (int u = 0; u < kChunkU; u++) k.v[u] = 0.0f;
+#pragma unroll
+    for (int u = 0; u < kChunkU / 2; u++) k.id2[u] = 0;
+    if ((ct & kPureChunk) || G >= total) return;  // (a pure chunk gets here in the checked build only)
+    uint32_t t = ct;
+    while (pre[t + 1] <= G) t++;
+    const uint4 r = rec[t];
+    const uint32_t q0 = r.x + 8u * G;
+    if (!checked(group_in_bounds(q0, ix.pcap), ix.err)) return;
+    load_ids8(ix.pid, q0, k.id2);
+    load_values8<DT>(ix.pval, q0, k.v);
+    k.w = __uint_as_float(r.w);
+    // at the segment's start or end the postings outside it weigh 0
+    const uint32_t lo = r.y > q0 ? r.y - q0 : 0u, hi = min(r.z - q0, (uint32_t)kChunkU);
+    k.lm = ((1u << hi) - 1u) & ~((1u << lo) - 1u);
+#pragma unroll
+    for (int u = 0; u < kChunkU; u++)
+        if (!((k.lm >> u) & 1u)) k.v[u] = 0.0f;
 }
 
 // Adds a lane's group to the window with shared-memory atomics (groups of different terms run at once and may
 // meet on a slot). Fixed point: each product (its weight carries the window's 2^e) is rounded to the nearest unit
 // and added with a native integer atomic; all 8 postings are added, those outside the segment as 0 at the slot
-// their load returned (an id of a neighbouring segment, or the zero padding: a valid slot, and an integer + 0
-// changes nothing), so the adds need no branch and no select.
+// their load returned (an id of a neighbouring segment, or 0: a valid slot, and an integer + 0 changes nothing),
+// so the adds need no branch and no select.
 template <bool FX>
 __device__ __forceinline__ void add_group(float* A, uint32_t lambda, uint32_t* err, const Group8& k) {
-    if (k.lm == 0) return;
 #pragma unroll
     for (int u = 0; u < kChunkU; u++) {
         const uint32_t slot = (k.id2[u >> 1] >> (16 * (u & 1))) & 0xFFFFu;
@@ -620,41 +640,47 @@ __device__ __forceinline__ void accumulate_groups(const DevIndex& ix, const uint
 }
 
 // The fixed-point window's e for a query of more terms than one table holds (its B must be known before the first
-// table's adds): a pass over all of them. Every thread of the block calls it; red is free on entry and on return.
+// table's adds), into red.fx_e: a pass over all of them. B is summed as a single table sums it (32 terms by
+// butterfly, then those sums in order), so e does not depend on the block shape. Every thread of the block calls it;
+// parts: kQueryTermLimit / 32 floats of scratch.
 template <int DT, int BLOCK>
-__device__ int window_scale_exp(const ScanArgs& a, uint32_t w, int64_t qb, int nt, TermRed<BLOCK / 32>& red) {
+__device__ void window_scale_exp(const ScanArgs& a, uint32_t w, int64_t qb, int nt, TermRed<BLOCK / 32>& red,
+                                 float* parts) {
     const DevIndex& ix = a.ix;
-    float b = 0.0f, m = 0.0f;
-    for (int t = threadIdx.x; t < nt; t += BLOCK) {
-        const int32_t j = a.q_indices[qb + t];
-        const float qv = a.q_values[qb + t];
-        if (j >= 0 && j < ix.dim && isfinite(qv) && list_in_bounds(j, w, ix.dim, ix.sigma)) {
-            const uint64_t sg = (uint64_t)j * ix.sigma + w;
-            if (ix.seg[sg + 1] != ix.seg[sg]) {
-                const float wq = fabsf((DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv);
-                b += wq * ix.vmax[j];
-                m = fmaxf(m, wq);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // (a query over the term limit is refused by the merge; its scan reads no terms past the limit's scratch)
+    const int groups = (min(nt, kQueryTermLimit) + 31) >> 5;
+    float m = 0.0f;
+    for (int g = warp; g < groups; g += BLOCK / 32) {
+        const int t = 32 * g + lane;
+        float b = 0.0f;
+        if (t < nt) {
+            const int32_t j = a.q_indices[qb + t];
+            const float qv = a.q_values[qb + t];
+            if (j >= 0 && j < ix.dim && isfinite(qv) && list_in_bounds(j, w, ix.dim, ix.sigma)) {
+                const uint64_t sg = (uint64_t)j * ix.sigma + w;
+                if (ix.seg[sg + 1] != ix.seg[sg]) {
+                    const float wq = fabsf((DT == SINDI_F8E4M3) ? qv * ix.scale[j] : qv);
+                    b = wq * ix.vmax[j];
+                    m = fmaxf(m, wq);
+                }
             }
         }
-    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        b += __shfl_xor_sync(kFull, b, o);
-        m = fmaxf(m, __shfl_xor_sync(kFull, m, o));
+        for (int o = 16; o > 0; o >>= 1) b += __shfl_xor_sync(kFull, b, o);
+        if (lane == 0) parts[g] = b;
     }
-    if ((threadIdx.x & 31) == 0) {
-        red.b[threadIdx.x >> 5] = b;
-        red.m[threadIdx.x >> 5] = __float_as_uint(m);
+    const uint32_t mw = __reduce_max_sync(kFull, __float_as_uint(m));
+    if (lane == 0) red.m[warp] = mw;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float B = 0.0f;
+        uint32_t M = 0;
+        for (int g = 0; g < groups; g++) B += parts[g];
+        for (int i = 0; i < BLOCK / 32; i++) M = max(M, red.m[i]);
+        red.fx_e = fx_exponent_from(B, __uint_as_float(M));
     }
     __syncthreads();
-    float B = 0.0f, M = 0.0f;
-    for (int i = 0; i < BLOCK / 32; i++) {
-        B += red.b[i];
-        M = fmaxf(M, __uint_as_float(red.m[i]));
-    }
-    const int e = fx_exponent_from(B, M);
-    __syncthreads();
-    return e;
 }
 
 // The term table of one query over one window for the pipelined scan, for terms c0 .. c0 + nc - 1 of the query (nc
@@ -748,25 +774,45 @@ __device__ __forceinline__ float key_floor_float(uint32_t k) {
     return order_bits_float(k);
 }
 
+// The running bound of a query as one window's cut compares with it.
+struct SlotBound {
+    uint32_t bits;  // least order bits of a score that can be in the answer
+    float thr;      // least score that counts
+    int32_t ithr;   // least fixed-point sum that counts
+};
+
+// From H's bin of the g-th emitted candidate. With skip_zero (every score of the query is >= 0 and the earlier
+// windows hold at least g slots, all with scores >= 0 and lower ids), a slot whose score is exactly 0 can never be
+// in the answer: when the bound reaches down to 0, only positive slots count. fx_e: the exponent of a fixed-point
+// window, else kNoFx.
+__device__ __forceinline__ SlotBound slot_bound(uint32_t bin, int32_t top, bool skip_zero, int fx_e) {
+    SlotBound b;
+    b.bits = hbin_floor(bin, top);
+    b.thr = key_floor_float(b.bits);
+    if (skip_zero && b.thr <= 0.0f) b.thr = __int_as_float(1);  // the least positive float (NaN stays NaN)
+    b.ithr = fx_e != kNoFx ? fx_threshold(b.thr, fx_e) : 0;
+    return b;
+}
+
 constexpr uint32_t kOneWarpEmits = 512;  // staged keys of a bounded window that one warp writes out alone
 
 // The cut of one accumulated window w of query row y: emits into the query's
 // candidate list every slot that can still be among its best g, and adds what
 // it emitted to the query's histogram H (ids >= N are not candidates).
 // `bounded`: g candidates of the query already exist with order bits of at
-// least `bound`; top: H's top bin (hbin_top). Every thread of the group S (NW
-// warps) calls it; the workspace must be free, and *cs.s_staged 0. LAST: the
-// scratch is not used again (a bounded cut then ends without a barrier).
+// least b.bits, and a slot counts when its score reaches b.thr, or its
+// fixed-point sum b.ithr; top: H's top bin (hbin_top). Every thread of the
+// group S (NW warps) calls it; the workspace must be free, and *cs.s_staged 0.
+// LAST: the scratch is not used again (a bounded cut then ends without a
+// barrier).
 template <typename S, int NW, bool FX = false, bool LAST = false>
-__device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t y, bool bounded, uint32_t bound,
-                              int32_t top, const CutScratch& cs, bool skip_zero = false, int fx_e = kNoFx) {
+__device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t y, bool bounded, const SlotBound& b,
+                              int32_t top, const CutScratch& cs, int fx_e = kNoFx) {
     constexpr int NT = S::kThreads;
     const DevIndex& ix = a.ix;
     const int tid = S::tid();
     const int lane = tid & 31, warp = tid >> 5;
-    uint32_t* hist = cs.hist;
     uint32_t* hist2 = cs.hist2;
-    uint32_t* warp_off = cs.warp_off;
     uint32_t* red = cs.red;
     uint32_t* st = cs.st;
     uint64_t* stage = reinterpret_cast<uint64_t*>(cs.region);
@@ -793,34 +839,42 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     };
     if (bounded) {
         // g candidates at or above the bound already exist, so only slots at or
-        // above it can be in the answer. With skip_zero (every score of the query
-        // is >= 0 and the earlier windows hold at least g slots, all with scores
-        // >= 0 and lower ids), a slot whose score is exactly 0 can never be
-        // either: when the bound reaches down to 0, only positive slots count.
-        // When the slots that can count fit the window's budget, emit all of
-        // them: no window histogram, no cut. One pass stages them (a shared
-        // counter: a few dozen a window), then one reservation for the group.
-        float thr = key_floor_float(bound);
-        if (skip_zero && thr <= 0.0f) thr = __int_as_float(1);  // the least positive float (NaN stays NaN)
+        // above it can be in the answer. When the slots that can count fit the
+        // window's budget, emit all of them: no window histogram, no cut. One
+        // pass stages them (a shared counter: a few dozen a window), then one
+        // reservation for the group.
+        const float thr = b.thr;
         const int n4 = (n_eff + 3) >> 2;
         const float4* A4 = reinterpret_cast<const float4*>(A);
         const int4* I4 = reinterpret_cast<const int4*>(A);
-        const int32_t ithr = fx ? fx_threshold(thr, fx_e) : 0;
-        // the window 4 slots per lane: one 16-byte load, a maximum and one compare; the per-slot work runs
-        // only for the rare lane that holds a candidate
+        const int32_t ithr = b.ithr;
+        // the window 4 slots per lane and load, four loads in flight; the per-slot work runs only for the
+        // rare lane that holds a candidate
         auto scan_bounded = [&](auto&& emit) {
             if (fx) {
-#pragma unroll 4
-                for (int i4 = tid; i4 < n4; i4 += NT) {
-                    const int4 x = I4[i4];
+                auto look = [&](const int4& x, int i) {
                     if (max(max(x.x, x.y), max(x.z, x.w)) >= ithr) {
-                        const int i = 4 * i4;
                         if (x.x >= ithr) emit(i);
                         if (x.y >= ithr && i + 1 < n_eff) emit(i + 1);
                         if (x.z >= ithr && i + 2 < n_eff) emit(i + 2);
                         if (x.w >= ithr && i + 3 < n_eff) emit(i + 3);
                     }
+                };
+                int i4 = tid;
+                for (; i4 + 3 * NT < n4; i4 += 4 * NT) {
+                    const int4 x = I4[i4], x1 = I4[i4 + NT], x2 = I4[i4 + 2 * NT], x3 = I4[i4 + 3 * NT];
+                    int32_t m = max(max(x.x, x.y), max(x.z, x.w));
+                    m = max(m, max(max(x1.x, x1.y), max(x1.z, x1.w)));
+                    m = max(m, max(max(x2.x, x2.y), max(x2.z, x2.w)));
+                    m = max(m, max(max(x3.x, x3.y), max(x3.z, x3.w)));
+                    if (m >= ithr) {
+                        look(x, 4 * i4);
+                        look(x1, 4 * (i4 + NT));
+                        look(x2, 4 * (i4 + 2 * NT));
+                        look(x3, 4 * (i4 + 3 * NT));
+                    }
                 }
+                for (; i4 < n4; i4 += NT) look(I4[i4], 4 * i4);
             } else {
 #pragma unroll 4
                 for (int i4 = tid; i4 < n4; i4 += NT) {
@@ -886,13 +940,15 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         }
         S::sync();
     }
-    // level 1: 12-bit bins of the score key. Each warp counts its slots in a
-    // private histogram of the 256 bins below the window's top bin (no
-    // contention between warps); the window histogram is their sum. When the
-    // cut falls below that range, a full 4096-bin histogram is used instead.
-    // the slot passes below read 4 slots per thread (thread t: slots 4 (t + k NT) .. + 3),
-    // and a warp's slots are the same in every pass
-    uint32_t* priv = reinterpret_cast<uint32_t*>(cs.region) + warp * kRelBins;
+    // level 1: 12-bit bins of the score key, in the 256 bins from the window's
+    // top bin down: the warps count in kCutHists histograms, the window's is
+    // their sum. When the cut falls below that range (32 octaves: in practice
+    // among the zeros of a window with few scored slots), the exact radix select
+    // decides instead. The scratch is small on purpose: three blocks of a
+    // 16,384-slot window fit an SM with it.
+    // the slot passes below read 4 slots per thread (thread t: slots 4 (t + k NT) .. + 3)
+    uint32_t* hists = reinterpret_cast<uint32_t*>(cs.region);
+    uint32_t* priv = hists + (warp % kCutHists) * kRelBins;
     const int n4w = (n_eff + 3) >> 2;
     const float4* A4w = reinterpret_cast<const float4*>(A);
     auto slots4 = [&](int i4, float v[4]) -> uint32_t {  // the group's scores; bit c: slot 4 i4 + c < n_eff
@@ -914,14 +970,13 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     }
     top_key = __reduce_max_sync(kFull, top_key);
     if (lane == 0) red[warp] = top_key;
-    for (int b = tid; b < kSubBins; b += NT) hist2[b] = 0;
+    for (int b = tid; b < kCutHists * kRelBins; b += NT) hists[b] = 0;
     S::sync();
     if (tid == 0) {
         uint32_t m = 0;
         for (int i = 0; i < NW; i++) m = max(m, red[i]);
         st[0] = m;
     }
-    for (int b = lane; b < kRelBins; b += 32) priv[b] = 0;
     S::sync();
     const uint32_t top_bin = st[0] >> (32 - kHistBits);
     for (int i4 = tid; i4 < n4w; i4 += NT) {
@@ -938,59 +993,28 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     S::sync();
     for (int b = tid; b < kRelBins; b += NT) {
         uint32_t c = 0;
-        for (int k = 0; k < NW; k++) c += reinterpret_cast<uint32_t*>(cs.region)[k * kRelBins + b];
-        cs.rel_hist[b] = c;  // slots in bin top_bin - b (b 255: that bin and all below)
+#pragma unroll
+        for (int k = 0; k < kCutHists; k++) c += hists[k * kRelBins + b];
+        hist2[b] = c;  // slots in bin top_bin - b (b 255: that bin and all below)
     }
     S::sync();
-    group_find_bin<kRelBins, S>([&](int b) { return cs.rel_hist[kRelBins - 1 - b]; }, g_w, red, st);
+    group_find_bin<kRelBins, S>([&](int b) { return hist2[kRelBins - 1 - b]; }, g_w, red, st);
     const uint32_t rel_cut = kRelBins - 1 - st[0];
-    uint32_t bw = top_bin - rel_cut;
-    uint32_t above_bw = st[1];
-    uint32_t c_bw = st[1] + st[2];  // slots in bins >= bw
-    S::sync();
+    const uint32_t bw = top_bin - rel_cut;
+    const uint32_t above_bw = st[1];
+    const uint32_t c_bw = st[1] + st[2];  // slots in bins >= bw
     const bool relative = rel_cut < (uint32_t)kRelBins - 1;
-    if (!relative) {
-        for (int b = tid; b < kHistBins; b += NT) hist[b] = 0;
-        S::sync();
-        for (int base = 0; base < n_eff; base += NT) {
-            const int i = base + tid;
-            const int bin = i < n_eff ? (int)(float_order_bits(A[i]) >> (32 - kHistBits)) : -1;
-            const unsigned peers = __match_any_sync(kFull, bin);
-            if (bin >= 0 && lane == __ffs(peers) - 1) atomicAdd(&hist[bin], (uint32_t)__popc(peers));
-        }
-        S::sync();
-        group_find_bin<kHistBins, S>([&](int b) { return hist[b]; }, g_w, red, st);
-        bw = st[0];
-        above_bw = st[1];
-        c_bw = st[1] + st[2];
-        S::sync();
-    }
+    S::sync();
+    for (int b = tid; b < kSubBins; b += NT) hist2[b] = 0;
+    if (tid == 0) *cs.s_staged = 0;
+    S::sync();
     wait_previous_kernels();  // the workspace is free from here on
     uint32_t lo = bw;
     // g slots already emitted at or above the bound prove the answer lies there
-    if (bounded) lo = max(lo, bound >> (32 - kHistBits));
+    if (bounded) lo = max(lo, b.bits >> (32 - kHistBits));
     const bool staged = relative && c_bw <= stage_cap;  // slots >= bin lo fit in the staging area
     uint32_t n_src = (uint32_t)n_eff;
     if (staged) {
-        // per-warp counts of slots at or above bin lo (from the private
-        // histograms) give every warp its staging range: no atomics below
-        uint32_t mine_w = 0;
-        for (int b = lane; b < kRelBins - 1; b += 32)
-            if (top_bin - (uint32_t)b >= lo) mine_w += priv[b];
-        mine_w = __reduce_add_sync(kFull, mine_w);
-        if (lane == 0) warp_off[warp] = mine_w;
-        S::sync();
-        if (tid == 0) {
-            uint32_t acc = 0;
-            for (int k = 0; k < NW; k++) {
-                const uint32_t c = warp_off[k];
-                warp_off[k] = acc;
-                acc += c;
-            }
-            cs.s_staged[0] = acc;
-        }
-        S::sync();  // the private histograms are dead from here on
-        uint32_t at = warp_off[warp];
         const unsigned lt = (1u << lane) - 1u;
         const float thr_lo = key_floor_float(lo << (32 - kHistBits));
         for (int b4 = warp * 32; b4 < n4w; b4 += NT) {
@@ -1004,12 +1028,20 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
                 m &= ok;
             }
             if (!__any_sync(kFull, m != 0u)) continue;
+            unsigned bal[4];
+            uint32_t cnt = 0;
 #pragma unroll
             for (int c = 0; c < 4; c++) {
-                const bool ok = (m >> c) & 1u;
-                const unsigned bal = __ballot_sync(kFull, ok);
-                if (ok) stage[at + __popc(bal & lt)] = key_of(4 * i4 + c);
-                at += __popc(bal);
+                bal[c] = __ballot_sync(kFull, (m >> c) & 1u);
+                cnt += (uint32_t)__popc(bal[c]);
+            }
+            uint32_t at = 0;
+            if (lane == 0) at = atomicAdd(cs.s_staged, cnt);
+            at = __shfl_sync(kFull, at, 0);
+#pragma unroll
+            for (int c = 0; c < 4; c++) {
+                if ((m >> c) & 1u) stage[at + __popc(bal[c] & lt)] = key_of(4 * i4 + c);
+                at += __popc(bal[c]);
             }
         }
         S::sync();
@@ -1018,8 +1050,8 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     // candidates: the staged keys, or the whole window
     auto src_key = [&](int i) -> uint64_t { return staged ? stage[i] : key_of(i); };
     uint64_t thr = (uint64_t)lo << kKeyBinShift;
-    bool exact = false;
-    if (lo == bw) {
+    bool exact = !relative;
+    if (relative && lo == bw) {
         // level 2: the next 8 bits, inside bin bw only
         for (int i = tid; i < (int)n_src; i += NT) {
             const uint64_t k = src_key(i);
@@ -1035,10 +1067,10 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         exact = c_cut > a.win_cap;
     }
     if (exact) {
-        // ties crowd the cut: exact best g_w of the window
+        // ties crowd the cut, or it lies far below the top: exact best g_w of the window
         thr = group_select_threshold<S>(src_key, (int)n_src, (int)g_w, hist2, st);
     }
-    if (bounded) thr = max(thr, (uint64_t)bound << 32);
+    if (bounded) thr = max(thr, (uint64_t)b.bits << 32);
     // emit keys >= thr: count, reserve the group's range with one atomic, write
     uint32_t mine = 0;
     for (int i = tid; i < (int)n_src; i += NT)
@@ -1058,8 +1090,11 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         const unsigned peers = __match_any_sync(kFull, bin);
         if (out && lane == __ffs(peers) - 1) atomicAdd(H + bin, (uint32_t)__popc(peers));
     }
-    S::sync();  // hist, region and st are reused by the caller's next cut
+    S::sync();  // hist2, region and st are reused by the caller's next cut
 }
+
+// Blocks of BLOCK threads an SM is to hold: about 1,024 threads in all (64 registers each).
+constexpr int scan_blocks_per_sm(int block) { return block == 384 ? 3 : 1024 / block; }
 
 // One block per (window, query): the term tables are staged in shared memory,
 // the block's warps scatter-add every term's postings of the window into A,
@@ -1068,30 +1103,30 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
 // histograms and staged candidates afterwards. The query's running bound is
 // found by one warp while the table's loads are in flight.
 // What bounds it: the SMs' issue slots and L1/shared data pipe (postings come
-// from L2). With chunks of one term each, a 12-bit H read by all threads and
-// a barrier per table step it took 126 instructions per 256 postings plus 14k
-// a block; 1,000 queries over 1M documents (16,384-slot windows): 3.59 ->
-// 2.74 ms a batch, over 8.8M (8,192 slots, FP16): 40.2 -> 27.8 ms, exact
-// search of uniform vectors (segments of 64 postings): 0.69 -> 0.40 ms.
+// from L2), and the barriers between its phases. With chunks of one term each,
+// a 12-bit H read by all threads, a barrier per table step and 37 KiB of
+// scratch beside every window (two blocks an SM at best), 1,000 queries over
+// 1M documents (16,384-slot windows) took 3.59 ms a batch, now 2.34; over 8.8M
+// (8,192 slots, FP16) 40.2, now 19.3; exact search of uniform vectors (segments
+// of 64 postings) 0.69, now 0.34.
 template <int DT, bool QUERY_MAJOR, int BLOCK, bool FX>
-__global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanArgs a) {
+__global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_kernel(ScanArgs a) {
     constexpr int kScanWarps = BLOCK / 32;
     constexpr int kTermChunk = BLOCK;   // query terms staged per pass (one per thread)
     using S = SyncBlock<BLOCK>;
     constexpr int kTableBytes = (16 * kTermChunk + (kTermChunk + 1) * 4 + kChunkTable * 2 + 15) & ~15;
-    constexpr int kPrivBytes = kScanWarps * kRelBins * 4;
-    constexpr int kCutBytes = kPrivBytes > kHistBins * 4 ? kPrivBytes : kHistBins * 4;
+    constexpr int kCutBytes = kCutHists * kRelBins * 4;
     constexpr int kRegionBytes = kTableBytes > kCutBytes ? kTableBytes : kCutBytes;
     extern __shared__ float A[];                    // [lambda]
     __shared__ __align__(16) unsigned char region[kRegionBytes];
-    __shared__ uint32_t rel_hist[kRelBins];
     __shared__ uint32_t hist2[kSubBins];
-    __shared__ uint32_t warp_off[kScanWarps];
     __shared__ uint32_t red[kScanWarps + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
     __shared__ uint32_t s_qneg;      // the query has a negative value
-    __shared__ uint32_t s_bound[2];  // H holds g candidates; the g-th's bin
+    __shared__ uint32_t s_bounded;   // H holds g candidates
+    __shared__ SlotBound s_bound;    // and what that means for this window
+    __shared__ int32_t s_top;        // H's top bin
     __shared__ TermRed<kScanWarps> tred;
     uint4* t_rec = reinterpret_cast<uint4*>(region);
     uint32_t* t_pre = reinterpret_cast<uint32_t*>(region + 16 * kTermChunk);
@@ -1110,6 +1145,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
     if (threadIdx.x == 0) {  // read after the term tables' barriers
         s_qneg = 0;
         s_staged = 0;
+        tred.qmax = 0;  // (written again only by this thread)
     }
     // the window is zeroed in two halves, while the query's offsets and then its terms are on their way
     float4* A4 = reinterpret_cast<float4*>(A);
@@ -1122,24 +1158,35 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
         qv = a.q_values[qb + threadIdx.x];
     }
     for (uint32_t m = n4h + threadIdx.x; m < n4; m += BLOCK) A4[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (a.use_partial == 1 && warp == kScanWarps - 1) {
-        // the histogram of what the query's earlier windows emitted (a snapshot:
-        // H only grows during the launch, so any snapshot bounds the answer)
+    // the query's running bound, by one warp: the bin of its g-th candidate in
+    // the histogram of what its earlier windows emitted (a snapshot: H only
+    // grows during the launch, so any snapshot bounds the answer)
+    constexpr int kBoundWarp = kScanWarps - 1;
+    bool found = false;
+    uint32_t bin = 0;
+    if (a.use_partial == 1 && warp == kBoundWarp) {
         wait_previous_kernels();  // the workspace is free from here on
-        uint32_t b = 0;
-        const bool f = warp_find_bound(H, a.g, &b);
-        if (lane == 0) {
-            s_bound[0] = f ? 1u : 0u;
-            s_bound[1] = b;
-        }
+        found = warp_find_bound(H, a.g, &bin);
     }
+    // what the bin means for this window (after the last term table's barriers)
+    auto publish_bound = [&]() {
+        if (lane != 0) return;
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(tred.qmax)));
+        s_top = top;
+        if (w == 0) {
+            wait_previous_kernels();
+            a.ws.qtop[y] = (uint32_t)top;
+        }
+        s_bounded = found ? 1u : 0u;
+        // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
+        const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
+        if (found) s_bound = slot_bound(bin, top, skip_zero, FX ? tred.fx_e : kNoFx);
+    };
 
     // fixed-point window: the unit 2^-e of this (query, window). B comes with the
     // term table when one table holds the query's terms, else from a pass of its own.
-    int fx_e = 0;
-    uint32_t qmax = 0;  // the query's largest product bound (bits)
     const bool fx_pre = FX && nt > kTermChunk;
-    if (fx_pre) fx_e = window_scale_exp<DT, BLOCK>(a, w, qb, nt, tred);
+    if (fx_pre) window_scale_exp<DT, BLOCK>(a, w, qb, nt, tred, reinterpret_cast<float*>(region));
     for (int c0 = 0; c0 == 0 || c0 < nt; c0 += kTermChunk) {
         const int nc = min(kTermChunk, nt - c0);
         if (c0) {
@@ -1149,9 +1196,14 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
             }
             __syncthreads();  // previous table fully consumed
         }
-        const uint32_t total = build_group_table<DT, BLOCK, FX>(a, w, j, qv, nc, t_rec, t_pre, c_term, tred, &s_qneg,
-                                                                fx_pre, fx_e, qmax);
-        accumulate_groups<DT, kScanWarps, FX>(ix, t_rec, t_pre, c_term, nc, total, warp, lane, A);
+        build_group_table<DT, BLOCK, FX>(a, w, j, qv, nc, t_rec, t_pre, c_term, tred, &s_qneg, fx_pre);
+        if (a.use_partial != 2 && warp == kBoundWarp && c0 + kTermChunk >= nt) publish_bound();
+        accumulate_groups<DT, kScanWarps, FX>(ix, t_rec, t_pre, c_term, nc, tred.total, warp, lane, A);
+    }
+    if (a.use_partial == 2 && warp == kBoundWarp) {
+        wait_previous_kernels();  // the first windows' candidates are all in H
+        found = warp_find_bound(H, a.g, &bin);
+        publish_bound();
     }
     __syncthreads();
 
@@ -1160,41 +1212,16 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) scan_window_kernel(ScanAr
     // accumulation
     allow_next_kernel();
 
-    const int32_t top = hbin_top(float_order_bits(__uint_as_float(qmax)));
-    if (w == 0 && threadIdx.x == 0) {
-        wait_previous_kernels();
-        a.ws.qtop[y] = (uint32_t)top;
-    }
-    bool bounded = false;
-    uint32_t bound = 0;  // order bits below which no slot can be in the answer, when g candidates exist
-    if (a.use_partial) {
-        if (a.use_partial == 2) {
-            if (warp == 0) {
-                wait_previous_kernels();  // the first windows' candidates are all in H
-                uint32_t b = 0;
-                const bool f = warp_find_bound(H, a.g, &b);
-                if (lane == 0) {
-                    s_bound[0] = f ? 1u : 0u;
-                    s_bound[1] = b;
-                }
-            }
-            __syncthreads();
-        }
-        bounded = s_bound[0] != 0;
-        bound = bounded ? hbin_floor(s_bound[1], top) : 0u;
-        wait_previous_kernels();
-    }
-    const CutScratch cs{reinterpret_cast<uint32_t*>(region), rel_hist, hist2, region, (uint32_t)kRegionBytes, warp_off,
-                        red, st, &s_staged};
-    // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
-    const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
+    const bool bounded = s_bounded != 0;
+    if (a.use_partial) wait_previous_kernels();
+    const CutScratch cs{hist2, region, (uint32_t)kRegionBytes, red, st, &s_staged};
+    const int fx_e = FX ? tred.fx_e : kNoFx;
     // a fixed-point window without a bound goes to FP32 for the full cut; a bounded one is read as integers
     if (FX && !bounded) {
         fx_window_to_float<S>(A, lambda, fx_e);
         S::sync();
     }
-    select_window<S, kScanWarps, FX, true>(a, A, w, y, bounded, bound, top, cs, skip_zero,
-                                           FX && bounded ? fx_e : kNoFx);
+    select_window<S, kScanWarps, FX, true>(a, A, w, y, bounded, s_bound, s_top, cs, bounded ? fx_e : kNoFx);
 }
 
 // ---------------------------------------------------------------------------
@@ -1233,10 +1260,7 @@ static size_t pipe_smem_bytes(uint32_t lambda) {
 template <int DT>
 __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) {
     extern __shared__ __align__(16) unsigned char dsm[];
-    __shared__ uint32_t hist[kHistBins];
-    __shared__ uint32_t rel_hist[kRelBins];
     __shared__ uint32_t hist2[kSubBins];
-    __shared__ uint32_t warp_off[kPipeCutWarps];
     __shared__ uint32_t red[kPipeCutWarps + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
@@ -1292,7 +1316,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
     }
 
     // ---- cut group: tables ahead, then the cut of every accumulated item
-    const CutScratch cs{hist, rel_hist, hist2, region, (uint32_t)kPipeRegionBytes, warp_off, red, st, &s_staged};
+    const CutScratch cs{hist2, region, (uint32_t)kPipeRegionBytes, red, st, &s_staged};
     uint32_t bi = 0;  // next stage to build: item bi, pass bp
     int bp = 0;
     auto build_next = [&](int t) {
@@ -1357,7 +1381,7 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
         }
         S::sync();
         const bool bounded = st[3] != 0;
-        const uint32_t bound = bounded ? hbin_floor(st[0], top) : 0u;
+        const SlotBound bound = slot_bound(bounded ? st[0] : 0u, top, false, kNoFx);
         S::sync();
         float* A = buf0 + (size_t)b * lam4;
         select_window<S, kPipeCutWarps>(a, A, w, y, bounded, bound, top, cs);
@@ -1440,10 +1464,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
     constexpr int NW = BLOCK / 32;
     using S = SyncBlock<BLOCK>;
     extern __shared__ __align__(16) unsigned char gsm[];
-    __shared__ uint32_t hist[kHistBins];
-    __shared__ uint32_t rel_hist[kRelBins];
     __shared__ uint32_t hist2[kSubBins];
-    __shared__ uint32_t warp_off[NW];
     __shared__ uint32_t red[NW + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
@@ -1603,8 +1624,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
 
     allow_next_kernel();
     wait_previous_kernels();  // the workspace (candidates, H) is free from here on
-    const CutScratch cs{hist, rel_hist, hist2, region, (uint32_t)group_region_bytes(BLOCK), warp_off, red, st,
-                        &s_staged};
+    const CutScratch cs{hist2, region, (uint32_t)group_region_bytes(BLOCK), red, st, &s_staged};
     for (uint32_t i = 0; i < qn; i++) {
         const uint32_t y = mrow[i];
         // the query's running bound: g candidates emitted at or above some bin (H only
@@ -1622,11 +1642,11 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
         }
         __syncthreads();
         const bool bounded = st[3] != 0;
-        const uint32_t bound = bounded ? hbin_floor(st[0], top) : 0u;
-        __syncthreads();
         // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
         const bool skip_zero = !((s_negmask >> i) & 1u) && ix.nonneg && (uint64_t)w * lambda >= sa.g;
-        select_window<S, NW>(sa, A + (size_t)i * lam4, w, y, bounded, bound, top, cs, skip_zero);
+        const SlotBound bound = slot_bound(bounded ? st[0] : 0u, top, skip_zero, kNoFx);
+        __syncthreads();
+        select_window<S, NW>(sa, A + (size_t)i * lam4, w, y, bounded, bound, top, cs);
     }
 }
 
@@ -2209,6 +2229,30 @@ static void launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t
     SINDI_CUDA(cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...));
 }
 
+// Threads of a window-scan block when the caller leaves the shape open, for windows of lambda slots and a launch of
+// `blocks` blocks. A block's phases (term table, adds, cut) each wait on something else, so an SM is kept busy by as
+// many blocks as its shared memory holds (4 * lambda + about 11 KiB each), at about 1,024 threads in all. Measured,
+// 1,000 queries over 1M documents, ms a batch by threads a block:
+//   lambda    128   256   384   512  1024
+//    4,096   2.70  3.33  3.87  4.90  8.25
+//    8,192   2.67  2.54  2.78  3.35  5.25
+//   12,000   2.79  2.34  2.49  2.83  4.20
+//   16,384   3.14  2.43  2.34  2.57  3.63
+//   32,768   6.88  4.21  3.61  3.13  2.86
+// (in the order of the table: 8, 4, 4, 3 and 1 blocks an SM are the best). A launch that leaves SMs idle anyway
+// takes larger blocks: with one window an SM, its threads are all there is to hide its latencies.
+static uint32_t default_scan_threads(uint32_t lambda, uint64_t blocks, uint32_t sms) {
+    const uint32_t bytes = 4 * window_stride(lambda);
+    uint32_t n = 1;  // blocks an SM holds
+    if (bytes <= 18 * 1024) n = 8;
+    else if (bytes <= 47 * 1024) n = 4;
+    else if (bytes <= 64 * 1024) n = 3;
+    else if (bytes <= 98 * 1024) n = 2;
+    if (blocks <= sms) n = 1;
+    else if (blocks <= 2 * (uint64_t)sms) n = n < 2 ? n : 2;
+    return n == 8 ? 128u : n == 4 ? 256u : n == 3 ? 384u : n == 2 ? 512u : 1024u;
+}
+
 template <int DT, bool QM, int BLOCK>
 static void allow_window_smem() {
     SINDI_CUDA(cudaFuncSetAttribute(scan_window_kernel<DT, QM, BLOCK, false>,
@@ -2221,10 +2265,14 @@ template <int DT>
 static void allow_window_smem_dt() {
     SINDI_CUDA(cudaFuncSetAttribute(scan_pipe_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)pipe_smem_bytes(kPipeMaxWindow)));
+    allow_window_smem<DT, false, 128>();
     allow_window_smem<DT, false, 256>();
+    allow_window_smem<DT, false, 384>();
     allow_window_smem<DT, false, 512>();
     allow_window_smem<DT, false, 1024>();
+    allow_window_smem<DT, true, 128>();
     allow_window_smem<DT, true, 256>();
+    allow_window_smem<DT, true, 384>();
     allow_window_smem<DT, true, 512>();
     allow_window_smem<DT, true, 1024>();
 }
@@ -2308,34 +2356,35 @@ static void launch_scan_t(const ScanArgs& a, uint32_t sigma, uint32_t nq, size_t
 }
 
 // Plain schedules (one query) take window-major grids; batched schedules take
-// query-major grids (window-major when sigma exceeds the grid's y limit). Both
-// default to 512-thread blocks.
+// query-major grids (window-major when sigma exceeds the grid's y limit).
 template <int DT, bool QM>
 static void launch_scan_block(uint32_t block, const ScanArgs& a, uint32_t sigma, uint32_t nq, size_t smem,
                               cudaStream_t s, bool pdl) {
-    if (block == 256) launch_scan_t<DT, QM, 256>(a, sigma, nq, smem, s, pdl);
+    if (block == 128) launch_scan_t<DT, QM, 128>(a, sigma, nq, smem, s, pdl);
+    else if (block == 256) launch_scan_t<DT, QM, 256>(a, sigma, nq, smem, s, pdl);
+    else if (block == 384) launch_scan_t<DT, QM, 384>(a, sigma, nq, smem, s, pdl);
     else if (block == 512) launch_scan_t<DT, QM, 512>(a, sigma, nq, smem, s, pdl);
     else launch_scan_t<DT, QM, 1024>(a, sigma, nq, smem, s, pdl);
 }
 
 template <int DT>
-static void launch_scan_dt(uint32_t block, bool batched, bool qm, const ScanArgs& a, uint32_t sigma, uint32_t nq,
-                           size_t smem, cudaStream_t s, bool pdl) {
-    if (block == 0) block = batched ? kScanThreadsBatched : kScanThreadsPlain;
+static void launch_scan_dt(uint32_t block, bool qm, const ScanArgs& a, uint32_t sigma, uint32_t nq, size_t smem,
+                           cudaStream_t s, bool pdl) {
     if (qm) launch_scan_block<DT, true>(block, a, sigma, nq, smem, s, pdl);
     else launch_scan_block<DT, false>(block, a, sigma, nq, smem, s, pdl);
 }
 
-static void launch_scan_pdl(int dt, uint32_t block, bool batched, bool qm, const ScanArgs& a, uint32_t sigma,
-                            uint32_t nq, size_t smem, cudaStream_t s, bool pdl) {
-    if (dt == SINDI_F32) launch_scan_dt<SINDI_F32>(block, batched, qm, a, sigma, nq, smem, s, pdl);
-    else if (dt == SINDI_F16) launch_scan_dt<SINDI_F16>(block, batched, qm, a, sigma, nq, smem, s, pdl);
-    else launch_scan_dt<SINDI_F8E4M3>(block, batched, qm, a, sigma, nq, smem, s, pdl);
+static void launch_scan_pdl(int dt, uint32_t block, bool qm, const ScanArgs& a, uint32_t sigma, uint32_t nq, size_t smem,
+                            cudaStream_t s, bool pdl) {
+    if (dt == SINDI_F32) launch_scan_dt<SINDI_F32>(block, qm, a, sigma, nq, smem, s, pdl);
+    else if (dt == SINDI_F16) launch_scan_dt<SINDI_F16>(block, qm, a, sigma, nq, smem, s, pdl);
+    else launch_scan_dt<SINDI_F8E4M3>(block, qm, a, sigma, nq, smem, s, pdl);
 }
 
 // The launches of one group of nq queries starting at row q0. `*chained` is
 // false for the first launch of a search call (it follows the caller's work
-// and must not overlap it) and true afterwards.
+// and must not overlap it) and true afterwards. in_flight: groups like this
+// one that run at once.
 struct QueryCsr {
     const int64_t* indptr;
     const int32_t* indices;
@@ -2345,7 +2394,8 @@ struct QueryCsr {
 static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& ws, const int64_t* q_indptr,
                          const int32_t* q_indices, const float* q_values, int64_t q0, uint32_t nq, bool batched,
                          uint32_t k, uint32_t* out_ids, float* out_scores, cudaStream_t stream, bool* chained,
-                         cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr, const QueryCsr* scan_q = nullptr) {
+                         cudaEvent_t ev0 = nullptr, cudaEvent_t ev1 = nullptr, const QueryCsr* scan_q = nullptr,
+                         uint32_t in_flight = 1) {
     configure_search_kernels(ix.device);
     const DevIndex dix = ix.dev();
     const size_t scan_smem = (size_t)window_stride(ix.lambda) * sizeof(float);
@@ -2358,7 +2408,10 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
     // the pipelined scan when asked for and its two window arrays fit; any
     // other shape is one block per window (block 0 or 1: the default size)
     const bool pipe = pl.block == SINDI_SCAN_PIPELINED && ix.lambda <= kPipeMaxWindow;
-    const uint32_t block = pl.block == SINDI_SCAN_PIPELINED ? 0u : pl.block;
+    const uint32_t block = pl.block > SINDI_SCAN_PIPELINED
+                               ? pl.block
+                               : default_scan_threads(ix.lambda, (uint64_t)nq * ix.sigma * in_flight,
+                                                      (uint32_t)device_sms(ix.device));
     const size_t pipe_smem = pipe_smem_bytes(ix.lambda);
     if (batched && !pipe && pl.group > 1 && ix.sigma <= 65535u) {
         // query groups: one block per (group, window); groups vary fastest, so the
@@ -2379,7 +2432,7 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
         // still enter the answer (the running bound of Alg. 2's heap, taken
         // from a block of windows instead of one window at a time).
         const uint32_t first = std::max<uint32_t>(2u, (ix.sigma + kSplitFraction - 1) / kSplitFraction);
-        launch_scan_pdl(ix.dtype, block, false, false, sa, first, nq, scan_smem, stream, *chained && !ev0);
+        launch_scan_pdl(ix.dtype, block, false, sa, first, nq, scan_smem, stream, *chained && !ev0);
         ScanArgs sb = sa;
         sb.use_partial = 2;
         sb.w0 = first;
@@ -2389,14 +2442,14 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
             const uint32_t blocks = (sb.nwin + kPlainPipeItems - 1) / kPlainPipeItems;
             launch_pipe(ix.dtype, sb, blocks, pipe_smem, stream, true);
         } else {
-            launch_scan_pdl(ix.dtype, block, false, false, sb, ix.sigma - first, nq, scan_smem, stream, true);
+            launch_scan_pdl(ix.dtype, block, false, sb, ix.sigma - first, nq, scan_smem, stream, true);
         }
         ix.launches += 1;
         ix.scan_launches += 1;
     } else {
         // query-major grids put the queries of one window next to each other
         // (shared lists stay in L2); gridDim.y limits sigma to 65535 there
-        launch_scan_pdl(ix.dtype, block, batched, batched && ix.sigma <= 65535u, sa, ix.sigma, nq, scan_smem,
+        launch_scan_pdl(ix.dtype, block, batched && ix.sigma <= 65535u, sa, ix.sigma, nq, scan_smem,
                         stream, *chained && !ev0);
     }
     if (ev1) SINDI_CUDA(cudaEventRecord(ev1, stream));
@@ -2436,7 +2489,7 @@ static void enqueue_plain_lanes(const IndexImpl& ix, const Plan& pl, const std::
         // one's last kernel runs; otherwise it follows that kernel's completion in stream order
         bool c = chain_queries && lane_chained[l] != 0;
         launch_group(ix, pl, wss[l], q_indptr, q_indices, q_values, q, 1, false, k, out_ids, out_scores, ls[l], &c,
-                     nullptr, nullptr, pruned);
+                     nullptr, nullptr, pruned, (uint32_t)lanes);
         lane_chained[l] = c ? 1 : 0;
     }
     for (cudaStream_t l : ls) {
