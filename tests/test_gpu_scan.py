@@ -65,3 +65,44 @@ def test_group_table_edges(n_terms, block, accum):
             assert len(set(ids[r])) == k
             np.testing.assert_allclose(sc[r], exact[ids[r]], rtol=TOL, atol=0, err_msg=f"{mode} {r}")
             np.testing.assert_allclose(sc[r], best, rtol=TOL, atol=0, err_msg=f"{mode} {r}")
+
+
+def _pattern(kind, n, rng):
+    """One value per document (0: not in the list), whole numbers: every sum below is exact in either window."""
+    base = rng.permutation(n).astype(np.int64) + 1
+    span = np.arange(n) // 128 % 8
+    if kind == "outside-the-sample":  # the best slots lie in spans the sampled cut does not read
+        return base + n * (span != 0)
+    if kind == "inside-the-sample":
+        return base + n * (span == 0)
+    if kind == "ascending":
+        return np.arange(1, n + 1)
+    if kind == "ties":
+        return np.full(n, 7)
+    if kind == "few-values":
+        return base % 3 + 1
+    assert kind == "rare"  # fewer scored documents than candidates
+    return np.where(rng.random(n) < 0.004, base, 0)
+
+
+@pytest.mark.parametrize("window", [300, 1024, 16384, 32768])
+@pytest.mark.parametrize("kind", ["outside-the-sample", "inside-the-sample", "ascending", "ties", "few-values", "rare"])
+def test_sampled_cuts_keep_the_exact_answer(kind, window):
+    n = 40_000
+    rng = np.random.default_rng(window)
+    v = _pattern(kind, n, rng)
+    has = v > 0
+    ip = np.concatenate([[0], np.cumsum(has)]).astype(np.int64)
+    t = [torch.from_numpy(a).to(DEV) for a in (ip, np.zeros(int(ip[-1]), np.int32), v[has].astype(np.float32))]
+    nq = 3
+    q = [torch.from_numpy(a).to(DEV) for a in (np.arange(nq + 1, dtype=np.int64), np.zeros(nq, np.int32),
+                                               np.array([1.0, 2.0, 0.5], np.float32))]
+    best = np.lexsort((np.arange(n), -v))  # score descending, then id
+    with sindi.Index(*t, 1, window=window) as idx:
+        for mode in ("plain", "batched"):
+            for k, gamma in ((1, 0), (10, 0), (600, 0), (10, 100), (1000, 3000)):
+                ids, sc = idx.search(*q, k=k, gamma=gamma, mode=mode)
+                idx.check()
+                for r, w in enumerate((1.0, 2.0, 0.5)):
+                    np.testing.assert_array_equal(ids[r].cpu().numpy(), best[:k], err_msg=f"{mode} {k} {gamma} {r}")
+                    np.testing.assert_array_equal(sc[r].cpu().numpy(), (w * v[best[:k]]).astype(np.float32))
