@@ -4,10 +4,11 @@
 //
 // Pipeline (one stream):
 //   validate_indptr  -> prune_select (warp per row) [+ prune_rows, prune_long_rows: rows that need a sort]
-//   -> exclusive scan of kept counts -> compact -> (window, dim) counts -> scan = seg
+//   -> exclusive scan of kept counts -> compact
 //   -> stable radix sort of kept entries by dim (input is in document order, so
 //      equal dims stay in ascending document id: the order is (dim, doc))
-//   -> [E4M3 per-list scales] -> pack (uint16 window-local id + value).
+//   -> (dim, window) counts -> scan = seg -> [List Pruning] -> [E4M3 per-list scales]
+//   -> order_pack (bank-aware order, uint16 window-local id + value, vmax, signs).
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
 
@@ -79,8 +80,7 @@ struct PruneArgs {
 // What bounds it: issue. A row of 120 entries takes about 450 warp
 // instructions, most of them in the bisection; a sorted row takes about 28
 // compare-exchange passes over shared memory and 2 * nnz dependent FP64 adds
-// by one lane (20.1 ms for 1M documents of 120 entries, alpha 0.5). Building
-// that index: 26.5 -> 7.4 ms.
+// by one lane (20.1 ms for 1M documents of 120 entries, alpha 0.5, now 1.6).
 // ---------------------------------------------------------------------------
 constexpr int kSelectWarps = 8;
 constexpr int kSelectRowCap = 512;
@@ -389,68 +389,93 @@ __global__ void __launch_bounds__(kLongBlock) prune_long_rows_kernel(PruneArgs p
     }
 }
 
-// Kept entries of every row -> compact arrays in document order (a warp per row).
-__global__ void compact_kernel(const int64_t* indptr, const int32_t* indices, const float* values, const uint32_t* mask,
-                               const int64_t* kept_off, int64_t n, uint32_t* sdim, uint32_t* sdoc, uint32_t* sval) {
+// Kept entries of every row -> compact arrays in document order: a warp per row, the row's mask words read at once.
+// Bound by HBM: the rows are read again, at 32-byte sectors (1M documents of 120 entries, 26 of them kept: 0.9 GB).
+constexpr int kCompactWarps = 8;
+__global__ void __launch_bounds__(kCompactWarps * 32) compact_kernel(const int64_t* indptr, const int32_t* indices,
+                                                                     const float* values, const uint32_t* mask,
+                                                                     const int64_t* kept_off, int64_t n, uint32_t* sdim,
+                                                                     uint32_t* sdoc, uint32_t* sval) {
     const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
-        const int64_t b = indptr[i], m = indptr[i + 1] - b;
-        const uint32_t* words = mask + keep_words(b, i);
-        int64_t o = kept_off[i];
-        for (int64_t t0 = 0; t0 < m; t0 += 32) {
-            const uint32_t kw = words[t0 >> 5];
+    const int64_t i = (int64_t)blockIdx.x * kCompactWarps + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const int64_t b = indptr[i], m = indptr[i + 1] - b;
+    const uint32_t* words = mask + keep_words(b, i);
+    int64_t o = kept_off[i];
+    const unsigned lt = (1u << lane) - 1u;
+    for (int64_t t0 = 0; t0 < m; t0 += 1024) {
+        const uint32_t mine = t0 + 32 * lane < m ? words[(t0 >> 5) + lane] : 0u;
+        const int nw = (int)(m - t0 < 1024 ? (m - t0 + 31) >> 5 : 32);
+#pragma unroll 4
+        for (int u = 0; u < nw; u++) {
+            const uint32_t kw = __shfl_sync(kFull, mine, u);
             if ((kw >> lane) & 1u) {
-                const int64_t at = o + __popc(kw & ((1u << lane) - 1u));
-                sdim[at] = (uint32_t)indices[b + t0 + lane];
+                const int64_t at = o + __popc(kw & lt);
+                const int64_t from = b + t0 + 32 * u + lane;
+                sdim[at] = (uint32_t)__ldg(indices + from);
                 sdoc[at] = (uint32_t)i;
-                sval[at] = __float_as_uint(values[b + t0 + lane]);
+                sval[at] = __float_as_uint(__ldg(values + from));
             }
             o += __popc(kw);
         }
     }
 }
 
-// Count postings of every list I_{j,w}: cnt[j * sigma + w].
-__global__ void list_count_kernel(const uint32_t* sdim, const uint32_t* sdoc, int64_t P, uint32_t lambda,
-                                  uint32_t sigma, uint32_t* cnt) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x)
-        atomicAdd(&cnt[(uint64_t)sdim[p] * sigma + sdoc[p] / lambda], 1u);
-}
-
-// Per-list E4M3 scale: max |x| over the list I_j (all windows) / 448.
-__global__ void list_scale_kernel(const uint32_t* seg, const uint32_t* sval, int32_t dim, uint32_t sigma,
-                                  float* scale) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t j = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); j < dim; j += warps) {
-        const uint32_t lo = seg[(uint64_t)j * sigma], hi = seg[(uint64_t)(j + 1) * sigma];
-        float amax = 0.0f;
-        for (uint32_t p = lo + lane; p < hi; p += 32) amax = fmaxf(amax, fabsf(__uint_as_float(sval[p])));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) amax = fmaxf(amax, __shfl_xor_sync(kFull, amax, o));
-        if (lane == 0) {
-            float sc = __fdiv_rn(amax, 448.0f);
-            scale[j] = sc > 0.0f ? sc : 1.0f;
+// Postings of every list I_{j,w}, cnt[j * sigma + w], from the sorted order (cnt zero on entry): a posting that starts
+// a list takes its place off the list's count, and adds it to the list that ends there (mod 2^32; the last list ends
+// at P). Two atomics a list instead of one a posting, whose head lists met on few addresses (26M: 574 -> 108 us).
+__global__ void list_count_kernel(const uint32_t* sdim, const uint32_t* sdoc, int64_t P, uint32_t lambda, uint32_t sigma,
+                                  uint32_t* cnt) {
+    auto list_of = [&](int64_t p) { return (uint64_t)sdim[p] * sigma + sdoc[p] / lambda; };
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
+        const uint64_t here = list_of(p);
+        if (p == P - 1) atomicAdd(&cnt[here], (uint32_t)P);
+        if (p > 0) {
+            const uint64_t before = list_of(p - 1);
+            if (before == here) continue;
+            atomicAdd(&cnt[before], (uint32_t)p);
         }
+        atomicSub(&cnt[here], (uint32_t)p);
     }
 }
 
-// Window-local ids and stored values.
+// amax[j] = the largest |x| of list I_j over all its windows, as the bits of a non-negative float (zero on entry):
+// a warp per list I_{j,w}.
+__global__ void list_amax_kernel(const uint32_t* seg, const uint32_t* sval, int64_t S, uint32_t sigma, uint32_t* amax) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t sg = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); sg < S; sg += warps) {
+        const uint32_t lo = seg[sg], hi = seg[sg + 1];
+        if (lo == hi) continue;
+        uint32_t m = 0;
+        for (uint32_t p = lo + lane; p < hi; p += 32) m = max(m, sval[p] & 0x7FFFFFFFu);
+        m = __reduce_max_sync(kFull, m);
+        if (lane == 0 && m > __ldcg(&amax[sg / sigma])) atomicMax(&amax[sg / sigma], m);
+    }
+}
+
+// Per-list E4M3 scale: max |x| over the list I_j (all windows) / 448.
+__global__ void list_scale_kernel(const uint32_t* amax, int32_t dim, float* scale) {
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < dim; j += (int64_t)gridDim.x * blockDim.x) {
+        const float sc = __fdiv_rn(__uint_as_float(amax[j]), 448.0f);
+        scale[j] = sc > 0.0f ? sc : 1.0f;
+    }
+}
+
+// A stored value: its code, and the value the scan reads back for it (without an E4M3 list's scale).
 template <int DT>
-__global__ void pack_kernel(const uint32_t* sdim, const uint32_t* sdoc, const uint32_t* sval, int64_t P,
-                            uint32_t lambda, const float* scale, uint16_t* pid, void* pval) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
-        pid[p] = (uint16_t)(sdoc[p] % lambda);
-        float v = __uint_as_float(sval[p]);
-        if (DT == SINDI_F32) {
-            static_cast<float*>(pval)[p] = v;
-        } else if (DT == SINDI_F16) {
-            static_cast<__half*>(pval)[p] = __float2half_rn(v);
-        } else {
-            float ratio = __fdiv_rn(v, scale[sdim[p]]);
-            static_cast<__nv_fp8_storage_t*>(pval)[p] = __nv_cvt_float_to_fp8(ratio, __NV_SATFINITE, __NV_E4M3);
-        }
+__device__ __forceinline__ float store_value(float v, float scale, void* pval, uint32_t p) {
+    if (DT == SINDI_F32) {
+        static_cast<float*>(pval)[p] = v;
+        return v;
+    } else if (DT == SINDI_F16) {
+        const __half h = __float2half_rn(v);
+        static_cast<__half*>(pval)[p] = h;
+        return __half2float(h);
+    } else {
+        const __nv_fp8_storage_t c = __nv_cvt_float_to_fp8(__fdiv_rn(v, scale), __NV_SATFINITE, __NV_E4M3);
+        static_cast<__nv_fp8_storage_t*>(pval)[p] = c;
+        return __half2float(__half(__nv_cvt_fp8_to_halfraw(c, __NV_E4M3)));
     }
 }
 
@@ -494,99 +519,135 @@ __global__ void lp_compact_kernel(const uint32_t* keep, const uint32_t* off, int
     }
 }
 
-// Posting order inside every list segment I_{j,w}, for the window scan's
+// The lists' final arrays: window ids and stored values of every segment I_{j,w}, in the order of the window scan's
 // shared-memory scatter-add: the 32 postings one add instruction of a warp
 // takes should sit in 32 different shared-memory banks (window slot mod 32),
 // which makes the shared-memory atomicAdd conflict-free. One warp per segment:
 //   1. every posting gets its bank b and a rank r among the segment's
 //      postings of bank b; ordering the postings by (r, b) visits the banks
 //      round robin, so any 32 consecutive ones hold 32 banks while every bank
-//      still has postings;
+//      still has postings. Its place is T[r] + the banks below b that hold
+//      more than r postings, T[r] = the postings of rank below r: one table
+//      row (T[r], the banks that hold more than r) per rank;
 //   2. that order is laid out over the positions of the segment in the order
 //      the scan's add instructions visit them (see kVecMin), so each
 //      instruction takes 32 consecutive ones.
 // Any order of a segment gives the same scores up to FP32 rounding; this one
 // only changes which bank each add of an instruction meets.
-// scratch: uint32[P]; (sdoc, sval) in, (odoc, oval) out.
+// The same pass packs the postings (uint16 id, stored value), raises the
+// list's largest |stored value| vmax[j] (bits; zero on entry) and sets *neg
+// when a stored value's sign bit is set. With those as passes of their own (a
+// warp per whole list for vmax) and 32 counts read per posting for its place,
+// 26M postings took 1.35 ms, now 0.53.
+// scratch: uint32[P], for segments longer than kOrderStage.
 constexpr int kOrderWarps = 8;
-__global__ void __launch_bounds__(kOrderWarps * 32) bank_order_kernel(const uint32_t* seg, int64_t S,
+constexpr uint32_t kOrderStage = 1024;  // postings of a segment whose order stays in shared memory
+constexpr uint32_t kOrderRanks = 256;   // ranks in the table; a segment with a fuller bank counts again per posting
+template <int DT>
+__global__ void __launch_bounds__(kOrderWarps * 32) order_pack_kernel(const uint32_t* seg, int64_t S, uint32_t sigma,
                                                                      const uint32_t* sdoc, const uint32_t* sval,
-                                                                     uint32_t lambda, uint32_t* scratch,
-                                                                     uint32_t* odoc, uint32_t* oval) {
-    __shared__ uint32_t cnt[kOrderWarps][32];
-    __shared__ uint32_t rnk[kOrderWarps][32];
+                                                                     uint32_t lambda, const float* scale,
+                                                                     uint32_t* scratch, uint16_t* pid, void* pval,
+                                                                     uint32_t* vmax, uint32_t* neg) {
+    __shared__ uint32_t s_cnt[kOrderWarps][32];
+    __shared__ uint32_t s_rnk[kOrderWarps][32];
+    __shared__ uint2 s_row[kOrderWarps][kOrderRanks];
+    __shared__ uint16_t s_perm[kOrderWarps][kOrderStage];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t *cnt = s_cnt[warp], *rnk = s_rnk[warp];
+    uint2* row = s_row[warp];
+    uint16_t* perm = s_perm[warp];
     const unsigned lt = (1u << lane) - 1u;
     const int64_t warps = (int64_t)gridDim.x * kOrderWarps;
+    uint32_t negative = 0;
     for (int64_t sg = (int64_t)blockIdx.x * kOrderWarps + warp; sg < S; sg += warps) {
         const uint32_t s = seg[sg], e = seg[sg + 1], L = e - s;
+        if (L == 0) continue;
+        const uint32_t j = (uint32_t)(sg / sigma);
+        const float sc = DT == SINDI_F8E4M3 ? scale[j] : 1.0f;
+        float top = 0.0f;
+        auto pack = [&](uint32_t p, uint32_t src) {
+            pid[p] = (uint16_t)(sdoc[src] % lambda);
+            const float v = store_value<DT>(__uint_as_float(sval[src]), sc, pval, p);
+            top = fmaxf(top, fabsf(v));
+            negative |= __float_as_uint(v) >> 31;
+        };
         if (L <= 32) {
             // one add instruction takes the whole segment: nothing to gain
-            if (lane < (int)L) {
-                odoc[s + lane] = sdoc[s + lane];
-                oval[s + lane] = sval[s + lane];
-            }
-            continue;
-        }
-        cnt[warp][lane] = 0;
-        rnk[warp][lane] = 0;
-        __syncwarp();
-        for (uint32_t i = lane; i < L; i += 32) atomicAdd(&cnt[warp][(sdoc[s + i] % lambda) & 31u], 1u);
-        __syncwarp();
-        for (uint32_t i0 = 0; i0 < L; i0 += 32) {
-            // rank = earlier postings of the same bank, in segment order (deterministic)
-            const uint32_t i = i0 + (uint32_t)lane;
-            const bool ok = i < L;
-            const uint32_t b = ok ? (sdoc[s + i] % lambda) & 31u : 32u + (uint32_t)lane;
-            const unsigned peers = __match_any_sync(kFull, b);
-            const uint32_t r = ok ? rnk[warp][b] + (uint32_t)__popc(peers & lt) : 0u;
-            __syncwarp();
-            if (ok && (peers & lt) == 0) rnk[warp][b] += (uint32_t)__popc(peers);
-            __syncwarp();
-            if (ok) {
-                // position of (r, b) in the (rank, bank) order
-                uint32_t q = 0;
-                for (uint32_t bb = 0; bb < 32; bb++) {
-                    const uint32_t c = cnt[warp][bb];
-                    q += c < r ? c : r;
-                    q += (bb < b && c > r) ? 1u : 0u;
-                }
-                scratch[s + q] = s + i;
-            }
-        }
-        __syncwarp();
-        // the positions in the order the scan's add instructions take them
-        uint32_t run = 0;
-        if (L >= kVecMin) {
-            const uint32_t g0 = s & ~7u, e8 = (e + 7u) & ~7u;
-            for (uint32_t base = g0; base < e8; base += (uint32_t)kChunkLen) {
-                for (int u = 0; u < kChunkU; u++) {
-                    const uint32_t p = base + 8u * (uint32_t)lane + (uint32_t)u;
-                    const bool ok = p >= s && p < e;
-                    const unsigned bal = __ballot_sync(kFull, ok);
-                    if (ok) {
-                        const uint32_t src = scratch[s + run + (uint32_t)__popc(bal & lt)];
-                        odoc[p] = sdoc[src];
-                        oval[p] = sval[src];
-                    }
-                    run += (uint32_t)__popc(bal);
-                }
-            }
+            if (lane < (int)L) pack(s + lane, s + lane);
         } else {
-            for (uint32_t u = 0; u * 32 < L; u++) {
-                const uint32_t p = s + 32u * u + (uint32_t)lane;
-                const bool ok = p < e;
+            cnt[lane] = 0;
+            rnk[lane] = 0;
+            __syncwarp();
+            for (uint32_t i = lane; i < L; i += 32) atomicAdd(&cnt[(sdoc[s + i] % lambda) & 31u], 1u);
+            __syncwarp();
+            const uint32_t mine = cnt[lane];
+            const uint32_t most = __reduce_max_sync(kFull, mine);
+            const bool table = most <= kOrderRanks;
+            if (table) {
+                uint32_t below = 0;
+                for (uint32_t r = 0; r < most; r++) {
+                    const unsigned more = __ballot_sync(kFull, mine > r);
+                    if (lane == 0) row[r] = make_uint2(below, more);
+                    below += (uint32_t)__popc(more);
+                }
+                __syncwarp();
+            }
+            const bool staged = L <= kOrderStage;
+            for (uint32_t i0 = 0; i0 < L; i0 += 32) {
+                // rank = earlier postings of the same bank, in segment order (deterministic)
+                const uint32_t i = i0 + (uint32_t)lane;
+                const bool ok = i < L;
+                const uint32_t b = ok ? (sdoc[s + i] % lambda) & 31u : 32u + (uint32_t)lane;
+                const unsigned peers = __match_any_sync(kFull, b);
+                const uint32_t r = ok ? rnk[b] + (uint32_t)__popc(peers & lt) : 0u;
+                __syncwarp();
+                if (ok && (peers & lt) == 0) rnk[b] += (uint32_t)__popc(peers);
+                __syncwarp();
+                if (ok) {
+                    // place of (r, b) in the (rank, bank) order
+                    uint32_t q = 0;
+                    if (table) {
+                        const uint2 t = row[r];
+                        q = t.x + (uint32_t)__popc(t.y & ((1u << b) - 1u));
+                    } else {
+                        for (uint32_t bb = 0; bb < 32; bb++) {
+                            const uint32_t c = cnt[bb];
+                            q += c < r ? c : r;
+                            q += (bb < b && c > r) ? 1u : 0u;
+                        }
+                    }
+                    if (staged) perm[q] = (uint16_t)i;
+                    else scratch[s + q] = i;
+                }
+            }
+            __syncwarp();
+            // the positions in the order the scan's add instructions take them
+            uint32_t run = 0;
+            auto lay = [&](uint32_t p, bool ok) {
                 const unsigned bal = __ballot_sync(kFull, ok);
                 if (ok) {
-                    const uint32_t src = scratch[s + run + (uint32_t)__popc(bal & lt)];
-                    odoc[p] = sdoc[src];
-                    oval[p] = sval[src];
+                    const uint32_t q = run + (uint32_t)__popc(bal & lt);
+                    pack(p, s + (staged ? (uint32_t)perm[q] : scratch[s + q]));
                 }
                 run += (uint32_t)__popc(bal);
+            };
+            if (L >= kVecMin) {
+                const uint32_t g0 = s & ~7u, e8 = (e + 7u) & ~7u;
+                for (uint32_t base = g0; base < e8; base += (uint32_t)kChunkLen)
+                    for (int u = 0; u < kChunkU; u++) {
+                        const uint32_t p = base + 8u * (uint32_t)lane + (uint32_t)u;
+                        lay(p, p >= s && p < e);
+                    }
+            } else {
+                for (uint32_t u = 0; u * 32 < L; u++) lay(s + 32u * u + (uint32_t)lane, s + 32u * u + (uint32_t)lane < e);
             }
+            __syncwarp();
         }
-        __syncwarp();
+        const uint32_t m = __reduce_max_sync(kFull, __float_as_uint(top));
+        if (lane == 0 && m > __ldcg(&vmax[j])) atomicMax(&vmax[j], m);
     }
+    if (__any_sync(kFull, negative != 0) && lane == 0) atomicOr(neg, 1u);
 }
 
 __global__ void fill_u32_kernel(float* p, int64_t n, float v) {
@@ -682,27 +743,16 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
     uint32_t* sdoc = P.alloc<uint32_t>(Pn);
     uint32_t* sval = P.alloc<uint32_t>(Pn);
     if (n > 0) {
-        compact_kernel<<<grid_for(n, 8, 152 * 32), 256, 0, stream>>>(ix.indptr, ix.indices, ix.values, mask, kept_off, n,
-                                                                     sdim, sdoc, sval);
+        compact_kernel<<<(unsigned)((n + kCompactWarps - 1) / kCompactWarps), kCompactWarps * 32, 0, stream>>>(
+            ix.indptr, ix.indices, ix.values, mask, kept_off, n, sdim, sdoc, sval);
         SINDI_CUDA(cudaGetLastError());
     }
     P.free(mask);
     P.free(kept_off);
 
     SINDI_TRACE_MSG("build_lists: compacted %lld kept entries", (long long)Pn);
-    // --- offsets of every list I_{j,w}
-    const int64_t S = (int64_t)d * sigma;
-    uint32_t* cnt = P.alloc<uint32_t>(S > 0 ? S : 1);
-    SINDI_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)(S > 0 ? S : 1), stream));
-    if (Pn > 0) {
-        list_count_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, Pn, lambda, sigma, cnt);
-        SINDI_CUDA(cudaGetLastError());
-    }
-    exclusive_scan<uint32_t, uint32_t>(cnt, ix.seg, S, P);
-    P.free(cnt);
-
-    SINDI_TRACE_MSG("build_lists: list offsets done");
     // --- stable sort by dim: (dim, doc) order
+    const int64_t S = (int64_t)d * sigma;
     {
         uint32_t* kb = P.alloc<uint32_t>(Pn);
         uint32_t* db = P.alloc<uint32_t>(Pn);
@@ -712,8 +762,21 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
         radix_sort_triples(sdim, sdoc, sval, kb, db, vb, Pn, bits, P);
         P.free(kb); P.free(db); P.free(vb);
     }
-
     SINDI_TRACE_MSG("build_lists: sort done");
+    // --- offsets of every list I_{j,w}
+    auto list_offsets = [&]() {
+        uint32_t* cnt = P.alloc<uint32_t>(S > 0 ? S : 1);
+        SINDI_CUDA(cudaMemsetAsync(cnt, 0, sizeof(uint32_t) * (size_t)(S > 0 ? S : 1), stream));
+        if (Pn > 0) {
+            list_count_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, Pn, lambda, sigma, cnt);
+            SINDI_CUDA(cudaGetLastError());
+        }
+        exclusive_scan<uint32_t, uint32_t>(cnt, ix.seg, S, P);
+        P.free(cnt);
+    };
+    list_offsets();
+    SINDI_TRACE_MSG("build_lists: list offsets done");
+
     if (lp > 0 && Pn > 0) {
         // --- List Pruning on the lists built so far, then their offsets again
         uint32_t* inv = P.alloc<uint32_t>(Pn);
@@ -746,14 +809,7 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
         sdoc = odoc;
         sval = oval;
         Pn = Pk;
-        uint32_t* cnt2 = P.alloc<uint32_t>(S > 0 ? S : 1);
-        SINDI_CUDA(cudaMemsetAsync(cnt2, 0, sizeof(uint32_t) * (size_t)(S > 0 ? S : 1), stream));
-        if (Pn > 0) {
-            list_count_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, Pn, lambda, sigma, cnt2);
-            SINDI_CUDA(cudaGetLastError());
-        }
-        exclusive_scan<uint32_t, uint32_t>(cnt2, ix.seg, S, P);
-        P.free(cnt2);
+        list_offsets();
         SINDI_TRACE_MSG("build_lists: list pruning kept %lld postings", (long long)Pn);
     }
     ix.postings = Pn;
@@ -768,45 +824,40 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
         SINDI_CUDA(cudaMemsetAsync(static_cast<uint8_t*>(ix.pval) + (size_t)Pn * ix.value_bytes(), 0,
                                    (size_t)(Pp - Pn) * ix.value_bytes(), stream));
     }
-    // --- values and window-local ids
+    // --- the lists: order, window-local ids, stored values, their bounds
+    ix.vmax = P.alloc<float>(d);
+    uint32_t* flags = P.alloc<uint32_t>((size_t)d + 1);  // largest |x| of every list; a stored value is negative
+    uint32_t* neg = flags + d;
+    SINDI_CUDA(cudaMemsetAsync(ix.vmax, 0, sizeof(float) * (size_t)d, stream));
+    SINDI_CUDA(cudaMemsetAsync(flags, 0, sizeof(uint32_t) * ((size_t)d + 1), stream));
     if (ix.dtype == SINDI_F8E4M3) {
-        if (d > 0) {
-            list_scale_kernel<<<grid_for(d, 8, 152 * 32), 256, 0, stream>>>(ix.seg, sval, d, sigma, ix.scale);
-            SINDI_CUDA(cudaGetLastError());
-        }
-    } else if (d > 0) {
+        list_amax_kernel<<<grid_for(S, 8, 152 * 32), 256, 0, stream>>>(ix.seg, sval, S, sigma, flags);
+        SINDI_CUDA(cudaGetLastError());
+        list_scale_kernel<<<grid_for(d, 256), 256, 0, stream>>>(flags, d, ix.scale);
+        SINDI_CUDA(cudaGetLastError());
+    } else {
         fill_u32_kernel<<<grid_for(d, 256), 256, 0, stream>>>(ix.scale, d, 1.0f);
         SINDI_CUDA(cudaGetLastError());
     }
     if (Pn > 0) {
-        // bank-aware order inside every segment (the scan's scatter-add)
         uint32_t* scratch = P.alloc<uint32_t>(Pn);
-        uint32_t* odoc = P.alloc<uint32_t>(Pn);
-        uint32_t* oval = P.alloc<uint32_t>(Pn);
-        bank_order_kernel<<<grid_for(S, kOrderWarps, 152 * 16), kOrderWarps * 32, 0, stream>>>(
-            ix.seg, S, sdoc, sval, lambda, scratch, odoc, oval);
-        SINDI_CUDA(cudaGetLastError());
+        const unsigned blocks = (unsigned)grid_for(S, kOrderWarps, 152 * 32);
+        uint32_t* vmax = reinterpret_cast<uint32_t*>(ix.vmax);
+        auto launch = [&](auto kern) {
+            kern<<<blocks, kOrderWarps * 32, 0, stream>>>(ix.seg, S, sigma, sdoc, sval, lambda, ix.scale, scratch, ix.pid,
+                                                          ix.pval, vmax, neg);
+            SINDI_CUDA(cudaGetLastError());
+        };
+        if (ix.dtype == SINDI_F32) launch(order_pack_kernel<SINDI_F32>);
+        else if (ix.dtype == SINDI_F16) launch(order_pack_kernel<SINDI_F16>);
+        else launch(order_pack_kernel<SINDI_F8E4M3>);
         P.free(scratch);
-        P.free(sdoc);
-        P.free(sval);
-        sdoc = odoc;
-        sval = oval;
-        if (ix.dtype == SINDI_F32)
-            pack_kernel<SINDI_F32><<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, sval, Pn, lambda, ix.scale,
-                                                                          ix.pid, ix.pval);
-        else if (ix.dtype == SINDI_F16)
-            pack_kernel<SINDI_F16><<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, sval, Pn, lambda, ix.scale,
-                                                                          ix.pid, ix.pval);
-        else
-            pack_kernel<SINDI_F8E4M3><<<grid_for(Pn, 256), 256, 0, stream>>>(sdim, sdoc, sval, Pn, lambda,
-                                                                             ix.scale, ix.pid, ix.pval);
-        SINDI_CUDA(cudaGetLastError());
     }
     P.free(sdim);
     P.free(sdoc);
     P.free(sval);
-    list_value_bounds(ix, stream);
-    ix.nonneg = postings_nonnegative(ix, stream);  // synchronises the stream
+    ix.nonneg = read_u32(neg, stream) == 0;  // synchronises the stream
+    P.free(flags);
     return SINDI_OK;
 }
 
