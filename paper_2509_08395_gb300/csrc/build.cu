@@ -480,27 +480,30 @@ __device__ __forceinline__ float store_value(float v, float scale, void* pval, u
 }
 
 // List Pruning (Sec. 4.1): every list I_j keeps its `lp` entries of largest
-// |x|, equal |x| by lower document id. Postings arrive in (dim, doc) order;
-// a stable sort by (dim, |x| descending) then ranks every entry in its list.
-// Sort keys: 0x7FFFFFFF - |x| bits (ascending = |x| descending), and the
-// entry's position.
-__global__ void lp_keys_kernel(const uint32_t* sval, int64_t P, uint32_t* inv, uint32_t* pos) {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < P; p += (int64_t)gridDim.x * blockDim.x) {
-        inv[p] = 0x7FFFFFFFu - (sval[p] & 0x7FFFFFFFu);
-        pos[p] = (uint32_t)p;
-    }
-}
-
-// Entry t of the (dim, |x| desc, doc asc) order has rank t - start(list) in
-// its list; the first lp survive. A dropped entry leaves its document's count.
-__global__ void lp_mark_kernel(const uint32_t* dim_sorted, const uint32_t* pos_sorted, int64_t P, const uint32_t* seg,
-                               uint32_t sigma, uint32_t lp, const uint32_t* sdoc, uint32_t* keep, uint32_t* kept) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < P; t += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t j = dim_sorted[t];
-        const uint32_t p = pos_sorted[t];
-        const bool k = (uint64_t)t - seg[(uint64_t)j * sigma] < lp;
-        keep[p] = k ? 1u : 0u;
-        if (!k) atomicSub(&kept[sdoc[p]], 1u);
+// |x|, equal |x| by lower document id. Postings are in (dim, doc) order, so a
+// list is one range and its order of documents the order of positions: a block
+// per list that is longer than lp selects the lp largest (|x|, position) keys.
+// A dropped entry leaves its document's count. (A stable sort of every posting
+// by |x| and dim, which ranked them all, took six radix passes.)
+constexpr int kLpBlock = 512;
+__global__ void __launch_bounds__(kLpBlock) lp_select_kernel(const uint32_t* seg, const uint32_t* sval, int32_t dim,
+                                                             uint32_t sigma, uint32_t lp, const uint32_t* sdoc,
+                                                             uint32_t* keep, uint32_t* kept) {
+    __shared__ uint32_t hist[256];
+    __shared__ uint32_t st[4];
+    for (int64_t j = blockIdx.x; j < dim; j += gridDim.x) {
+        const uint32_t lo = seg[(uint64_t)j * sigma], L = seg[(uint64_t)(j + 1) * sigma] - lo;
+        uint64_t T = 0;
+        auto key_of = [&](int64_t i) -> uint64_t {
+            return ((uint64_t)(sval[lo + i] & 0x7FFFFFFFu) << 32) | (0xFFFFFFFFu - (uint32_t)i);
+        };
+        if (L > lp) T = group_select_threshold<SyncBlock<kLpBlock>>(key_of, (int64_t)L, (int64_t)lp, hist, st);
+        for (int64_t i = threadIdx.x; i < L; i += kLpBlock) {
+            const bool k = key_of(i) >= T;
+            keep[lo + i] = k ? 1u : 0u;
+            if (!k) atomicSub(&kept[sdoc[lo + i]], 1u);
+        }
+        __syncthreads();
     }
 }
 
@@ -779,22 +782,9 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
 
     if (lp > 0 && Pn > 0) {
         // --- List Pruning on the lists built so far, then their offsets again
-        uint32_t* inv = P.alloc<uint32_t>(Pn);
-        uint32_t* dcp = P.alloc<uint32_t>(Pn);
-        uint32_t* pos = P.alloc<uint32_t>(Pn);
-        uint32_t* kb = P.alloc<uint32_t>(Pn);
-        uint32_t* db = P.alloc<uint32_t>(Pn);
-        uint32_t* vb = P.alloc<uint32_t>(Pn);
-        lp_keys_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(sval, Pn, inv, pos);
-        SINDI_CUDA(cudaGetLastError());
-        SINDI_CUDA(cudaMemcpyAsync(dcp, sdim, sizeof(uint32_t) * (size_t)Pn, cudaMemcpyDeviceToDevice, stream));
-        radix_sort_triples(inv, dcp, pos, kb, db, vb, Pn, 31, P);  // by |x| descending (stable)
-        int bits = 0;
-        while (bits < 32 && ((uint64_t)1 << bits) < (uint64_t)d) bits++;
-        radix_sort_triples(dcp, inv, pos, kb, db, vb, Pn, bits, P);  // then by dim (stable)
-        uint32_t* keep = kb;  // scratch reuse
+        uint32_t* keep = P.alloc<uint32_t>(Pn);
         uint32_t* off = P.alloc<uint32_t>(Pn + 1);
-        lp_mark_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(dcp, pos, Pn, ix.seg, sigma, lp, sdoc, keep, kept);
+        lp_select_kernel<<<grid_for(d, 1, 152 * 4), kLpBlock, 0, stream>>>(ix.seg, sval, d, sigma, lp, sdoc, keep, kept);
         SINDI_CUDA(cudaGetLastError());
         exclusive_scan<uint32_t, uint32_t>(keep, off, Pn, P);
         const int64_t Pk = read_u32(off + Pn, stream);
@@ -803,7 +793,7 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
         uint32_t* oval = P.alloc<uint32_t>(Pk > 0 ? Pk : 1);
         lp_compact_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(keep, off, Pn, sdim, sdoc, sval, odim, odoc, oval);
         SINDI_CUDA(cudaGetLastError());
-        P.free(inv); P.free(dcp); P.free(pos); P.free(kb); P.free(db); P.free(vb); P.free(off);
+        P.free(keep); P.free(off);
         P.free(sdim); P.free(sdoc); P.free(sval);
         sdim = odim;
         sdoc = odoc;

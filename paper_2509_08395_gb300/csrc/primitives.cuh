@@ -303,12 +303,13 @@ inline void radix_sort_triples(uint32_t* key_a, uint32_t* doc_a, uint32_t* val_a
 // 1 <= g <= n, returns T such that exactly g keys are >= T. The leading bits
 // all keys share are found first (one max/min reduction) and skipped; 8-bit
 // digits then go from the highest differing bit down, and a digit bucket that
-// holds exactly the remainder ends the search early.
+// holds exactly the remainder ends the search early. N: int, or int64_t for
+// arrays that may be longer.
 //   hist: shared uint32[256]; st: shared uint32[4].
 // Every thread of the group must call it (it synchronises).
 // ---------------------------------------------------------------------------
-template <typename S, typename KeyOf>
-__device__ uint64_t group_select_threshold(const KeyOf& key_of, int n, int g, uint32_t* hist, uint32_t* st) {
+template <typename S, typename KeyOf, typename N>
+__device__ uint64_t group_select_threshold(const KeyOf& key_of, N n, N g, uint32_t* hist, uint32_t* st) {
     constexpr int BLOCK = S::kThreads;
     constexpr int W = BLOCK / 32;
     static_assert(2 * W * 2 <= 256, "scratch for the reduction lives in hist");
@@ -316,7 +317,7 @@ __device__ uint64_t group_select_threshold(const KeyOf& key_of, int n, int g, ui
     const int lane = tid & 31, warp = tid >> 5;
     // shared prefix: highest bit where the largest and smallest key differ
     uint64_t mx = 0, mn = ~0ull;
-    for (int i = tid; i < n; i += BLOCK) {
+    for (N i = tid; i < n; i += BLOCK) {
         const uint64_t k = key_of(i);
         mx = k > mx ? k : mx;
         mn = k < mn ? k : mn;
@@ -354,8 +355,8 @@ __device__ uint64_t group_select_threshold(const KeyOf& key_of, int n, int g, ui
     for (int shift = hb - 7 > 0 ? hb - 7 : 0;; shift = shift - 8 > 0 ? shift - 8 : 0) {
         for (int b = tid; b < 256; b += BLOCK) hist[b] = 0;
         S::sync();
-        for (int base = 0; base < n; base += BLOCK) {
-            int i = base + tid;
+        for (N base = 0; base < n; base += BLOCK) {
+            const N i = base + tid;
             int dig = -1;
             if (i < n) {
                 uint64_t k = key_of(i);
