@@ -406,17 +406,28 @@ __global__ void __launch_bounds__(kCompactWarps * 32) compact_kernel(const int64
     for (int64_t t0 = 0; t0 < m; t0 += 1024) {
         const uint32_t mine = t0 + 32 * lane < m ? words[(t0 >> 5) + lane] : 0u;
         const int nw = (int)(m - t0 < 1024 ? (m - t0 + 31) >> 5 : 32);
-#pragma unroll 4
-        for (int u = 0; u < nw; u++) {
-            const uint32_t kw = __shfl_sync(kFull, mine, u);
-            if ((kw >> lane) & 1u) {
-                const int64_t at = o + __popc(kw & lt);
-                const int64_t from = b + t0 + 32 * u + lane;
-                sdim[at] = (uint32_t)__ldg(indices + from);
-                sdoc[at] = (uint32_t)i;
-                sval[at] = __float_as_uint(__ldg(values + from));
+        for (int u0 = 0; u0 < nw; u0 += 4) {  // four words' loads in flight
+            uint32_t kw[4], jj[4], xx[4];
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                kw[u] = __shfl_sync(kFull, mine, u0 + u);  // (0 past the row)
+                const int64_t from = b + t0 + 32 * (u0 + u) + lane;
+                jj[u] = xx[u] = 0;
+                if ((kw[u] >> lane) & 1u) {
+                    jj[u] = (uint32_t)__ldg(indices + from);
+                    xx[u] = __float_as_uint(__ldg(values + from));
+                }
             }
-            o += __popc(kw);
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                if ((kw[u] >> lane) & 1u) {
+                    const int64_t at = o + __popc(kw[u] & lt);
+                    sdim[at] = jj[u];
+                    sdoc[at] = (uint32_t)i;
+                    sval[at] = xx[u];
+                }
+                o += __popc(kw[u]);
+            }
         }
     }
 }
@@ -541,14 +552,16 @@ __global__ void lp_compact_kernel(const uint32_t* keep, const uint32_t* off, int
 // list's largest |stored value| vmax[j] (bits; zero on entry) and sets *neg
 // when a stored value's sign bit is set. With those as passes of their own (a
 // warp per whole list for vmax) and 32 counts read per posting for its place,
-// 26M postings took 1.35 ms, now 0.53.
+// 26M postings took 1.35 ms, now 0.50.
 // scratch: uint32[P], for segments longer than kOrderStage.
 constexpr int kOrderWarps = 8;
+static_assert(kVecMin <= 33, "segments of more than 32 postings are tiled on 8-aligned groups");
 constexpr uint32_t kOrderStage = 1024;  // postings of a segment whose order stays in shared memory
 constexpr uint32_t kOrderRanks = 256;   // ranks in the table; a segment with a fuller bank counts again per posting
 template <int DT>
 __global__ void __launch_bounds__(kOrderWarps * 32) order_pack_kernel(const uint32_t* seg, int64_t S, uint32_t sigma,
-                                                                     const uint32_t* sdoc, const uint32_t* sval,
+                                                                     const uint32_t* __restrict__ sdoc,
+                                                                     const uint32_t* __restrict__ sval,
                                                                      uint32_t lambda, const float* scale,
                                                                      uint32_t* scratch, uint16_t* pid, void* pval,
                                                                      uint32_t* vmax, uint32_t* neg) {
@@ -569,20 +582,21 @@ __global__ void __launch_bounds__(kOrderWarps * 32) order_pack_kernel(const uint
         const uint32_t j = (uint32_t)(sg / sigma);
         const float sc = DT == SINDI_F8E4M3 ? scale[j] : 1.0f;
         float top = 0.0f;
-        auto pack = [&](uint32_t p, uint32_t src) {
-            pid[p] = (uint16_t)(sdoc[src] % lambda);
-            const float v = store_value<DT>(__uint_as_float(sval[src]), sc, pval, p);
+        auto put = [&](uint32_t p, uint32_t doc, uint32_t val) {
+            pid[p] = (uint16_t)(doc % lambda);
+            const float v = store_value<DT>(__uint_as_float(val), sc, pval, p);
             top = fmaxf(top, fabsf(v));
             negative |= __float_as_uint(v) >> 31;
         };
         if (L <= 32) {
             // one add instruction takes the whole segment: nothing to gain
-            if (lane < (int)L) pack(s + lane, s + lane);
+            if (lane < (int)L) put(s + lane, __ldg(sdoc + s + lane), __ldg(sval + s + lane));
         } else {
             cnt[lane] = 0;
             rnk[lane] = 0;
             __syncwarp();
-            for (uint32_t i = lane; i < L; i += 32) atomicAdd(&cnt[(sdoc[s + i] % lambda) & 31u], 1u);
+#pragma unroll 4
+            for (uint32_t i = lane; i < L; i += 32) atomicAdd(&cnt[(__ldg(sdoc + s + i) % lambda) & 31u], 1u);
             __syncwarp();
             const uint32_t mine = cnt[lane];
             const uint32_t most = __reduce_max_sync(kFull, mine);
@@ -597,12 +611,14 @@ __global__ void __launch_bounds__(kOrderWarps * 32) order_pack_kernel(const uint
                 __syncwarp();
             }
             const bool staged = L <= kOrderStage;
+            uint32_t next = __ldg(sdoc + s + lane);  // (L > 32)
             for (uint32_t i0 = 0; i0 < L; i0 += 32) {
                 // rank = earlier postings of the same bank, in segment order (deterministic)
                 const uint32_t i = i0 + (uint32_t)lane;
                 const bool ok = i < L;
-                const uint32_t b = ok ? (sdoc[s + i] % lambda) & 31u : 32u + (uint32_t)lane;
-                const unsigned peers = __match_any_sync(kFull, b);
+                const uint32_t b = (next % lambda) & 31u;
+                if (i + 32 < L) next = __ldg(sdoc + s + i + 32);
+                const unsigned peers = warp_match<5>(b) & __ballot_sync(kFull, ok);
                 const uint32_t r = ok ? rnk[b] + (uint32_t)__popc(peers & lt) : 0u;
                 __syncwarp();
                 if (ok && (peers & lt) == 0) rnk[b] += (uint32_t)__popc(peers);
@@ -627,23 +643,32 @@ __global__ void __launch_bounds__(kOrderWarps * 32) order_pack_kernel(const uint
             __syncwarp();
             // the positions in the order the scan's add instructions take them
             uint32_t run = 0;
-            auto lay = [&](uint32_t p, bool ok) {
-                const unsigned bal = __ballot_sync(kFull, ok);
-                if (ok) {
-                    const uint32_t q = run + (uint32_t)__popc(bal & lt);
-                    pack(p, s + (staged ? (uint32_t)perm[q] : scratch[s + q]));
-                }
-                run += (uint32_t)__popc(bal);
-            };
-            if (L >= kVecMin) {
+            {
                 const uint32_t g0 = s & ~7u, e8 = (e + 7u) & ~7u;
-                for (uint32_t base = g0; base < e8; base += (uint32_t)kChunkLen)
+                for (uint32_t base = g0; base < e8; base += (uint32_t)kChunkLen) {
+                    // the chunk's eight gathers in flight
+                    const uint32_t p0 = base + 8u * (uint32_t)lane;
+                    uint32_t src[kChunkU], doc[kChunkU], val[kChunkU];
+#pragma unroll
                     for (int u = 0; u < kChunkU; u++) {
-                        const uint32_t p = base + 8u * (uint32_t)lane + (uint32_t)u;
-                        lay(p, p >= s && p < e);
+                        const bool ok = p0 + u >= s && p0 + u < e;
+                        const unsigned bal = __ballot_sync(kFull, ok);
+                        const uint32_t q = run + (uint32_t)__popc(bal & lt);
+                        src[u] = ok ? s + (staged ? (uint32_t)perm[q] : scratch[s + q]) : 0xFFFFFFFFu;
+                        run += (uint32_t)__popc(bal);
                     }
-            } else {
-                for (uint32_t u = 0; u * 32 < L; u++) lay(s + 32u * u + (uint32_t)lane, s + 32u * u + (uint32_t)lane < e);
+#pragma unroll
+                    for (int u = 0; u < kChunkU; u++) {
+                        doc[u] = val[u] = 0;
+                        if (src[u] != 0xFFFFFFFFu) {
+                            doc[u] = __ldg(sdoc + src[u]);
+                            val[u] = __ldg(sval + src[u]);
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < kChunkU; u++)
+                        if (src[u] != 0xFFFFFFFFu) put(p0 + u, doc[u], val[u]);
+                }
             }
             __syncwarp();
         }
