@@ -52,6 +52,15 @@ cudaMemPool_t library_pool(int device) {
     return pool;
 }
 
+// Returns a build's temporaries to the system, all but kPoolReserve bytes beyond what is in use: mapping and unmapping
+// them took 1 of the 4 ms an index of 1M documents is built in when indexes are built one after another.
+constexpr uint64_t kPoolReserve = (uint64_t)1 << 30;
+static void trim_pool(cudaMemPool_t pool) {
+    uint64_t used = 0;
+    SINDI_CUDA(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used));
+    SINDI_CUDA(cudaMemPoolTrimTo(pool, (size_t)(used + kPoolReserve)));
+}
+
 enum class Where { Host, Device, Invalid };
 
 static Where where_is(const void* p) {
@@ -323,7 +332,7 @@ sindi_status sindi_build(const int64_t* indptr, const int32_t* indices, const fl
         sindi_status st = build_lists(ix, s);
         SINDI_TRACE_MSG("sindi_build: lists done, status %d", (int)st);
         SINDI_CUDA(cudaStreamSynchronize(s));
-        SINDI_CUDA(cudaMemPoolTrimTo(ix.pool, 0));
+        trim_pool(ix.pool);
         if (st != SINDI_OK) {
             free_index_memory(ix, s);
             delete h;
