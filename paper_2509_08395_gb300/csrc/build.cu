@@ -65,22 +65,26 @@ struct PruneArgs {
 // per lane in registers. The kept set is a prefix of the pi order (|x|
 // descending, equal |x| by lower dim), so only its last |x|, K, is needed:
 // the largest K whose entries of |x| >= K reach alpha * mass (or vn entries).
-// K is found by bisecting the bit patterns of |x|, both ends pulled to the
-// nearest |x| of the row after every step (7 to 9 steps for 128 entries).
+// K is found by bisecting the bit patterns of |x|, the end that moves pulled to
+// the nearest |x| of the row (about 6 steps for 128 entries). The steps compare
+// 32-bit sums (the shares' top 31 bits: one warp reduction a step); the K they
+// end at is then checked with the whole sums, and moved when it is not the one.
 //
 // The rule sums FP64 values one after another in pi order. The values are
 // FP32, so unless their magnitudes spread over 2^20 or more, every such sum
-// is exact and does not depend on the order: with all |x| whole multiples of
-// 2^low and their sum below 2^(low + 53), the sums are taken here as 64-bit
-// integers in units of 2^low, and the kept count is bit-identical. Rows for
+// is exact and does not depend on the order: with the least |x|'s last place
+// as the unit and the sum below 2^53 units, the sums are taken here as whole
+// numbers of units, and the kept count is bit-identical. Rows for
 // which this does not hold, rows whose dims do not ascend (their duplicates
 // need a sort to be found) and rows of more than 512 entries go to
 // prune_rows_kernel.
 //
-// What bounds it: issue. A row of 120 entries takes about 450 warp
-// instructions, most of them in the bisection; a sorted row takes about 28
-// compare-exchange passes over shared memory and 2 * nnz dependent FP64 adds
-// by one lane (20.1 ms for 1M documents of 120 entries, alpha 0.5, now 1.6).
+// What bounds it: issue, and the chain of warp reductions. The row lengths are
+// split over three launches (up to 128, 256, 512 entries): with all of them in
+// one kernel the unrolled paths did not fit the instruction cache, and warps
+// waited 6.5 of 14 cycles per instruction for it. Sorting a row instead takes
+// 28 compare-exchange passes over shared memory and 2 * nnz dependent FP64 adds
+// by one lane (20.1 ms for 1M documents of 120 entries, alpha 0.5; now 1.48).
 // ---------------------------------------------------------------------------
 constexpr int kSelectWarps = 8;
 constexpr int kSelectRowCap = 512;
@@ -118,73 +122,102 @@ __device__ __forceinline__ bool prune_row_select(const PruneArgs& p, int64_t i, 
     }
     if (!__all_sync(kFull, ascending)) return false;
     uint32_t nz_l = 0, top_l = 0, least_l = 0xFFFFFFFFu;
-    int low_l = 1 << 20;
 #pragma unroll
     for (int u = 0; u < I; u++) {
-        if (a[u]) {
-            nz_l++;
-            top_l = max(top_l, a[u]);
-            least_l = min(least_l, a[u]);
-            const int E = max(1, (int)(a[u] >> 23));
-            const uint32_t mant = a[u] >= 0x800000u ? (a[u] & 0x7FFFFFu) | 0x800000u : a[u];
-            low_l = min(low_l, E + __ffs(mant) - 1);
-        }
+        nz_l += a[u] ? 1u : 0u;
+        top_l = max(top_l, a[u]);
+        least_l = a[u] ? min(least_l, a[u]) : least_l;
     }
     const uint32_t nz = __reduce_add_sync(kFull, nz_l);
     uint32_t K = 1, ties = 0xFFFFFFFFu;  // kept: |x| > K, and the first `ties` entries of |x| == K
     const bool by_mass = p.vn == 0;
     if (nz && (by_mass ? p.alpha < 1.0 : p.vn < nz)) {
         const uint32_t top = __reduce_max_sync(kFull, top_l);
-        const int low = by_mass ? __reduce_min_sync(kFull, low_l) : 0;
-        // every |x| is a multiple of 2^low and below 2^(Etop + 24) (both offset by 150)
+        const uint32_t least = __reduce_min_sync(kFull, least_l);
+        // every |x| is a whole number of units 2^(low - 150), below 2^(Etop + 24 - low) of them
+        const int low = max(1, (int)(least >> 23));
         if (by_mass && max(1, (int)(top >> 23)) + 24 + (32 - __clz((int)(nz - 1) | 1)) - low > 53) return false;
-        // an entry's share: |x| in units of 2^low, or 1 when entries are counted
+        // an entry's share: |x| in units (the shift is at most 29), or 1 when entries are counted
         auto share = [&](uint32_t x) -> uint64_t {
-            if (!by_mass) return 1;
-            const int E = max(1, (int)(x >> 23));
-            const uint64_t mant = x >= 0x800000u ? (x & 0x7FFFFFu) | 0x800000u : x;
-            return E >= low ? mant << (E - low) : mant >> (low - E);
+            if (!by_mass) return x ? 1u : 0u;
+            const uint32_t mant = x >= 0x800000u ? (x & 0x7FFFFFu) | 0x800000u : x;
+            const int sh = x ? max(1, (int)(x >> 23)) - low : 0;
+            return ((uint64_t)__funnelshift_l(mant, 0u, sh) << 32) | (mant << sh);
         };
-        uint64_t f[I];
         uint64_t mine = 0;
 #pragma unroll
-        for (int u = 0; u < I; u++) {
-            f[u] = a[u] ? share(a[u]) : 0;
-            mine += f[u];
-        }
+        for (int u = 0; u < I; u++) mine += share(a[u]);
+        const uint64_t mass = warp_sum53(mine);
         uint64_t target = p.vn;
         if (by_mass) {
-            const uint64_t mass = warp_sum53(mine);
             target = (uint64_t)ceil(__dmul_rn(p.alpha, (double)mass));  // prefix >= alpha * mass, for whole prefixes
             if (target == 0) target = 1;
         }
-        // lo: the least |x| known to reach the target with everything above it; hi: K < hi
-        uint32_t lo = __reduce_min_sync(kFull, least_l), hi = top + 1;
-        while (lo + 1 < hi) {
-            const uint32_t mid = lo + (hi - lo) / 2;  // lo < mid < hi
-            uint64_t s = 0;
-            uint32_t up = 0xFFFFFFFFu, down = 0;  // the nearest |x| of the row at or above mid, and below it
+        const int cutoff = max(0, 33 - __clzll((long long)mass));  // at most 22; mass >> cutoff below 2^31
+        const uint32_t target32 = (uint32_t)(target >> cutoff);
+        uint32_t s32[I];
 #pragma unroll
-            for (int u = 0; u < I; u++) {
-                const bool ge = a[u] >= mid;
-                s += ge ? f[u] : 0ull;
-                up = ge ? min(up, a[u]) : up;
-                down = ge ? down : max(down, a[u]);
-            }
-            if (warp_sum53(s) >= target) {
+        for (int u = 0; u < I; u++) {
+            const uint64_t f = share(a[u]);
+            s32[u] = __funnelshift_r((uint32_t)f, (uint32_t)(f >> 32), cutoff);
+        }
+        // lo: the least |x| whose entries and those above it reach the target; hi: K < hi (both by the short sums)
+        uint32_t lo = least, hi = top + 1;
+        uint32_t s_lo = (uint32_t)(mass >> cutoff), s_hi = 0;  // about the sums at and above lo and hi
+        bool half = false;
+        while (lo + 1 < hi) {
+            // by turns where the target lies between the two sums, and halfway
+            uint32_t off = (hi - lo) / 2;
+            if (!half && s_lo > s_hi && s_lo > target32)
+                off = (uint32_t)(__fdividef((float)(s_lo - target32), (float)(s_lo - s_hi)) * (float)(hi - lo));
+            half = !half;
+            const uint32_t mid = lo + min(max(off, 1u), hi - lo - 1u);  // lo < mid < hi
+            uint32_t sum = 0;
+#pragma unroll
+            for (int u = 0; u < I; u++) sum += a[u] >= mid ? s32[u] : 0u;
+            sum = __reduce_add_sync(kFull, sum);
+            if (sum >= target32) {
+                s_lo = sum;
+                uint32_t up = 0xFFFFFFFFu;  // the nearest |x| of the row at or above mid
+#pragma unroll
+                for (int u = 0; u < I; u++) up = a[u] >= mid ? min(up, a[u]) : up;
                 lo = __reduce_min_sync(kFull, up);
             } else {
+                s_hi = sum;
+                uint32_t down = 0;  // and below it
+#pragma unroll
+                for (int u = 0; u < I; u++) down = a[u] < mid ? max(down, a[u]) : down;
                 hi = __reduce_max_sync(kFull, down) + 1;
             }
         }
         K = lo;
-        uint64_t above = 0;
+        while (true) {
+            uint64_t above_l = 0;
+            uint32_t eq_l = 0;
 #pragma unroll
-        for (int u = 0; u < I; u++) above += a[u] > K ? f[u] : 0ull;
-        above = warp_sum53(above);
-        const uint64_t fk = share(K);
-        // most rows: one entry of |x| == K, needed whole (target > above by the choice of K)
-        ties = target - above <= fk ? 1u : (uint32_t)((target - above + fk - 1) / fk);
+            for (int u = 0; u < I; u++) {
+                above_l += share(a[u] > K ? a[u] : 0u);
+                eq_l += a[u] == K ? 1u : 0u;
+            }
+            const uint64_t above = warp_sum53(above_l);
+            const uint32_t eq = __reduce_add_sync(kFull, eq_l);
+            const uint64_t fk = share(K);
+            if (above >= target) {  // K lies higher
+                uint32_t up = 0xFFFFFFFFu;
+#pragma unroll
+                for (int u = 0; u < I; u++) up = a[u] > K ? min(up, a[u]) : up;
+                K = __reduce_min_sync(kFull, up);
+            } else if (above + eq * fk < target) {  // lower (some |x| does reach the target: alpha < 1, vn < nz)
+                uint32_t down = 0;
+#pragma unroll
+                for (int u = 0; u < I; u++) down = a[u] < K ? max(down, a[u]) : down;
+                K = __reduce_max_sync(kFull, down);
+            } else {
+                // most rows: one entry of |x| == K, needed whole
+                ties = target - above <= fk ? 1u : (uint32_t)((target - above + fk - 1) / fk);
+                break;
+            }
+        }
     }
     uint32_t r = 0, tied = 0;
     uint32_t* words = p.mask + keep_words(b, i);
@@ -203,26 +236,35 @@ __device__ __forceinline__ bool prune_row_select(const PruneArgs& p, int64_t i, 
     return true;
 }
 
-__global__ void __launch_bounds__(kSelectWarps * 32) prune_select_kernel(PruneArgs p) {
+// Rows of more than `over` and at most 32 * I entries: a warp takes `rows` (<= 32) consecutive ones. The first launch
+// (over < 0) also lists the rows that no launch takes.
+template <int I>
+__global__ void __launch_bounds__(kSelectWarps * 32, I <= 8 ? 4 : 2) prune_select_kernel(PruneArgs p, int over, int rows) {
     const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * kSelectWarps + (threadIdx.x >> 5);
-    if (i >= p.n) return;
-    const int64_t b = p.indptr[i];
-    const int64_t m = p.indptr[i + 1] - b;
-    bool done;
-    if (m <= 64) done = prune_row_select<2>(p, i, b, (int)m, lane);
-    else if (m <= 128) done = prune_row_select<4>(p, i, b, (int)m, lane);
-    else if (m <= 256) done = prune_row_select<8>(p, i, b, (int)m, lane);
-    else if (m <= kSelectRowCap) done = prune_row_select<16>(p, i, b, (int)m, lane);
-    else done = false;
-    if (done || lane != 0) return;
-    if (m > kMaxRowNnz) {
-        atomicOr(p.err, kErrDocTooLong);
-        p.kept[i] = 0;
-    } else if (m > kPruneRowCap) {
-        p.long_rows[atomicAdd(p.n_long, 1u)] = (uint32_t)i;
-    } else {
-        p.sort_rows[atomicAdd(p.n_sort, 1u)] = (uint32_t)i;
+    const int64_t i0 = ((int64_t)blockIdx.x * kSelectWarps + (threadIdx.x >> 5)) * rows;
+    int64_t b_l = 0, m_l = -1;  // lane l: row i0 + l
+    if (lane < rows && i0 + lane < p.n) {
+        b_l = p.indptr[i0 + lane];
+        m_l = p.indptr[i0 + lane + 1] - b_l;
+    }
+    if (over < 0 && m_l > kSelectRowCap) {
+        if (m_l > kMaxRowNnz) {
+            atomicOr(p.err, kErrDocTooLong);
+            p.kept[i0 + lane] = 0;
+        } else if (m_l > kPruneRowCap) {
+            p.long_rows[atomicAdd(p.n_long, 1u)] = (uint32_t)(i0 + lane);
+        } else {
+            p.sort_rows[atomicAdd(p.n_sort, 1u)] = (uint32_t)(i0 + lane);
+        }
+    }
+    unsigned todo = __ballot_sync(kFull, m_l > over && m_l >= 0 && m_l <= 32 * I);
+    while (todo) {
+        const int l = __ffs(todo) - 1;
+        todo &= todo - 1u;
+        const int64_t b = __shfl_sync(kFull, b_l, l);
+        const int m = (int)__shfl_sync(kFull, m_l, l);
+        if (!prune_row_select<I>(p, i0 + l, b, m, lane) && lane == 0)
+            p.sort_rows[atomicAdd(p.n_sort, 1u)] = (uint32_t)(i0 + l);
     }
 }
 
@@ -738,7 +780,14 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
     if (n > 0) {
         const PruneArgs pa{ix.indptr, ix.indices, ix.values, n,         d,          ix.alpha,      vn,
                            kept,      mask,       left_rows, n_left,    left_rows + n, n_left + 1, ix.err};
-        prune_select_kernel<<<(unsigned)((n + kSelectWarps - 1) / kSelectWarps), kSelectWarps * 32, 0, stream>>>(pa);
+        // rows per warp: as many as leave four waves of warps
+        const int rows = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (152 * 32 * 4)));
+        const unsigned blocks = (unsigned)((n + (int64_t)rows * kSelectWarps - 1) / ((int64_t)rows * kSelectWarps));
+        prune_select_kernel<4><<<blocks, kSelectWarps * 32, 0, stream>>>(pa, -1, rows);
+        SINDI_CUDA(cudaGetLastError());
+        prune_select_kernel<8><<<blocks, kSelectWarps * 32, 0, stream>>>(pa, 128, rows);
+        SINDI_CUDA(cudaGetLastError());
+        prune_select_kernel<16><<<blocks, kSelectWarps * 32, 0, stream>>>(pa, 256, rows);
         SINDI_CUDA(cudaGetLastError());
         // the listed rows; their counts stay on the device
         prune_rows_kernel<<<grid_for(n, kPruneWarps, 152 * 6), kPruneWarps * 32, 0, stream>>>(pa);
