@@ -1161,8 +1161,8 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
     S::sync();  // hist2, region and st are reused by the caller's next cut
 }
 
-// Blocks of BLOCK threads an SM is to hold: about 1,024 threads in all (64 registers each).
-constexpr int scan_blocks_per_sm(int block) { return block == 384 ? 3 : 1024 / block; }
+// Blocks of BLOCK threads an SM is to hold: about 1,024 threads in all (56 to 64 registers each).
+constexpr int scan_blocks_per_sm(int block) { return block == 384 ? 3 : block == 224 ? 5 : 1024 / block; }
 
 // One block per (window, query): the term tables are staged in shared memory,
 // the block's warps scatter-add every term's postings of the window into A,
@@ -1179,6 +1179,7 @@ constexpr int scan_blocks_per_sm(int block) { return block == 384 ? 3 : 1024 / b
 // of 64 postings) 0.69, now 0.34.
 template <int DT, bool QUERY_MAJOR, int BLOCK, bool FX>
 __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_kernel(ScanArgs a) {
+    static_assert(BLOCK % 32 == 0, "whole warps: the per-warp arrays have BLOCK / 32 entries");
     constexpr int kScanWarps = BLOCK / 32;
     constexpr int kTermChunk = BLOCK;   // query terms staged per pass (one per thread)
     using S = SyncBlock<BLOCK>;
@@ -2335,25 +2336,28 @@ static void launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t
 // Threads of a window-scan block when the caller leaves the shape open, for windows of lambda slots and a launch of
 // `blocks` blocks. A block's phases (term table, adds, cut) each wait on something else, so an SM is kept busy by as
 // many blocks as its shared memory holds (4 * lambda + about 11 KiB each), at about 1,024 threads in all. Measured,
-// 1,000 queries over 1M documents, ms a batch by threads a block:
-//   lambda    128   256   384   512  1024
-//    4,096   2.70  3.33  3.87  4.90  8.25
-//    8,192   2.67  2.54  2.78  3.35  5.25
-//   12,000   2.79  2.34  2.49  2.83  4.20
-//   16,384   3.14  2.43  2.34  2.57  3.63
-//   32,768   6.88  4.21  3.61  3.13  2.86
-// (in the order of the table: 8, 4, 4, 3 and 1 blocks an SM are the best). A launch that leaves SMs idle anyway
-// takes larger blocks: with one window an SM, its threads are all there is to hide its latencies.
+// 1,000 queries over 1M documents, ms a batch by threads a block (the second row with a faster rerank):
+//   lambda    128   224   256   384   512  1024
+//    4,096   2.70  3.06  3.33  3.87  4.90  8.25
+//    8,192         2.25  2.35
+//    8,192   2.67  2.46  2.54  2.78  3.35  5.25
+//   12,000   2.79  2.42  2.34  2.49  2.83  4.20
+//   16,384   3.14  2.60  2.43  2.34  2.57  3.63
+//   32,768   6.88  4.89  4.21  3.61  3.13  2.86
+// (in the order of the table: 8, 5, 5, 4, 3 and 1 blocks an SM are the best; 200 queries over 8.8M documents of FP16
+// postings at 8,192: 256 threads 3.76, 224 3.51). A launch that leaves SMs idle anyway takes larger blocks: with one
+// window an SM, its threads are all there is to hide its latencies.
 static uint32_t default_scan_threads(uint32_t lambda, uint64_t blocks, uint32_t sms) {
     const uint32_t bytes = 4 * window_stride(lambda);
     uint32_t n = 1;  // blocks an SM holds
     if (bytes <= 18 * 1024) n = 8;
+    else if (bytes <= 36 * 1024) n = 5;
     else if (bytes <= 47 * 1024) n = 4;
     else if (bytes <= 64 * 1024) n = 3;
     else if (bytes <= 98 * 1024) n = 2;
     if (blocks <= sms) n = 1;
     else if (blocks <= 2 * (uint64_t)sms) n = n < 2 ? n : 2;
-    return n == 8 ? 128u : n == 4 ? 256u : n == 3 ? 384u : n == 2 ? 512u : 1024u;
+    return n == 8 ? 128u : n == 5 ? 224u : n == 4 ? 256u : n == 3 ? 384u : n == 2 ? 512u : 1024u;
 }
 
 template <int DT, bool QM, int BLOCK>
@@ -2369,11 +2373,13 @@ static void allow_window_smem_dt() {
     SINDI_CUDA(cudaFuncSetAttribute(scan_pipe_kernel<DT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)pipe_smem_bytes(kPipeMaxWindow)));
     allow_window_smem<DT, false, 128>();
+    allow_window_smem<DT, false, 224>();
     allow_window_smem<DT, false, 256>();
     allow_window_smem<DT, false, 384>();
     allow_window_smem<DT, false, 512>();
     allow_window_smem<DT, false, 1024>();
     allow_window_smem<DT, true, 128>();
+    allow_window_smem<DT, true, 224>();
     allow_window_smem<DT, true, 256>();
     allow_window_smem<DT, true, 384>();
     allow_window_smem<DT, true, 512>();
@@ -2465,6 +2471,7 @@ template <int DT, bool QM>
 static void launch_scan_block(uint32_t block, const ScanArgs& a, uint32_t sigma, uint32_t nq, size_t smem,
                               cudaStream_t s, bool pdl) {
     if (block == 128) launch_scan_t<DT, QM, 128>(a, sigma, nq, smem, s, pdl);
+    else if (block == 224) launch_scan_t<DT, QM, 224>(a, sigma, nq, smem, s, pdl);
     else if (block == 256) launch_scan_t<DT, QM, 256>(a, sigma, nq, smem, s, pdl);
     else if (block == 384) launch_scan_t<DT, QM, 384>(a, sigma, nq, smem, s, pdl);
     else if (block == 512) launch_scan_t<DT, QM, 512>(a, sigma, nq, smem, s, pdl);
@@ -2693,7 +2700,9 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
     const bool batched = prm.mode == SINDI_MODE_BATCHED;
     int64_t chunk = 1;
     if (batched) {
-        const size_t budget = (size_t)1 << 31;  // 2 GiB of workspace per launch group
+        // workspace per launch group: every group reads the lists again and ends in a wave that is not full (1,000
+        // queries over 8.8M documents: 2 GiB 18.85 ms, 4 GiB 18.39)
+        const size_t budget = (size_t)4 << 30;
         const size_t per_query = workspace_bytes(1, pl.cand_cap, pl.fcap, pl.top_cap);
         chunk = std::max<int64_t>(1, std::min<int64_t>(n_queries, (int64_t)(budget / per_query)));
         chunk = std::min<int64_t>(chunk, 65535);
