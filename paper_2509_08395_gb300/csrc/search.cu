@@ -49,7 +49,8 @@ constexpr int kPlainLanes = 24;            // plain schedule: query chains in fl
 constexpr int kGraphLanes = 56;            // and in a recorded graph, at most (graph_lanes)
 constexpr uint32_t kPlainPipeItems = 6;    // plain schedule, pipelined scan: windows per block
 constexpr uint32_t kSplitMinWindows = 8;   // plain schedule: a query of this many windows or more scans
-constexpr uint32_t kSplitFraction = 8;     // its first 1/kSplitFraction windows first
+constexpr uint32_t kSplitFraction = 8;     // its first 1/kSplitFraction windows first; a batch does the same while
+constexpr uint64_t kSplitWaves = 6;        // its blocks fill the device fewer times than this
 constexpr int kMaxScanWarps = 1024 / 32;   // largest scan block
 constexpr int kChunkTable = 1024;          // chunks mapped to their list by a table (then a search)
 constexpr int kHistBits = 12;              // a window cut's bins: the top 12 bits of a score key
@@ -1289,9 +1290,19 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
         const int64_t rest = ix.n_docs - (int64_t)w * lambda;
         const int n_eff = (int)(rest < (int64_t)lambda ? rest : (int64_t)lambda);
         const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
-        sample_cut<BLOCK, FX>(A, n_eff, min(a.g, (uint32_t)n_eff), s_top, skip_zero, fx_e,
-                              reinterpret_cast<uint32_t*>(region), &s_bound);
-        direct = s_bound.need != ~0u;
+        if ((uint32_t)n_eff <= a.win_cap) {
+            // the window's budget holds all its slots (a deep pool over a small window): no cut to look for
+            if (threadIdx.x == 0) {
+                s_bound = slot_bound(0, s_top, skip_zero, fx_e);
+                s_bound.bits = 0;
+            }
+            __syncthreads();
+            direct = true;
+        } else {
+            sample_cut<BLOCK, FX>(A, n_eff, min(a.g, (uint32_t)n_eff), s_top, skip_zero, fx_e,
+                                  reinterpret_cast<uint32_t*>(region), &s_bound);
+            direct = s_bound.need != ~0u;
+        }
     }
     select_window<S, kScanWarps, FX, true>(a, A, w, y, direct, s_bound, s_top, cs, fx_e);
 }
@@ -2279,7 +2290,7 @@ __global__ void pad_results_kernel(uint32_t* out_ids, float* out_scores, int64_t
 // Sizes of one search: candidates per query and the buffers that follow.
 struct Plan {
     bool final_stage;
-    uint32_t g, win_cap, cand_cap, fcap, top_cap, merge_blocks, block;
+    uint32_t g, win_cap, cand_cap, fcap, top_cap, block;
     uint32_t group;  // batched scan: queries per block (1 = one block per (query, window))
     bool fixed;      // the one-block-per-window scan accumulates in fixed point
 };
@@ -2306,9 +2317,6 @@ static Plan make_plan(const IndexImpl& ix, const sindi_search_params& prm) {
     while (f < 2 * p.g && f < 16384) f <<= 1;
     p.fcap = f;
     p.top_cap = p.final_stage ? 1 : p.g;
-    // two blocks: a query's merge is one block unless its candidates crowd the cut, and every block of
-    // the grid is resident (holding its shared memory) while the scan finishes
-    p.merge_blocks = std::max<uint32_t>(1, std::min<uint32_t>(2, p.cand_cap / 8192));
     p.block = prm.block_threads;
     p.group = group_size(ix, prm.group, prm.block_threads);
     p.fixed = prm.accumulator == SINDI_ACCUM_FIXED32 || (prm.accumulator == SINDI_ACCUM_AUTO && !p.final_stage);
@@ -2346,19 +2354,18 @@ static void launch_kernel(void (*kern)(Params...), dim3 grid, dim3 block, size_t
 //   16,384   3.14  2.60  2.43  2.34  2.57  3.63
 //   32,768   6.88  4.89  4.21  3.61  3.13  2.86
 // (in the order of the table: 8, 5, 5, 4, 3 and 1 blocks an SM are the best; 200 queries over 8.8M documents of FP16
-// postings at 8,192: 256 threads 3.76, 224 3.51). A launch that leaves SMs idle anyway takes larger blocks: with one
-// window an SM, its threads are all there is to hide its latencies.
-static uint32_t default_scan_threads(uint32_t lambda, uint64_t blocks, uint32_t sms) {
+// postings at 8,192: 256 threads 3.76, 224 3.51). A launch of fewer blocks takes larger ones, 1,024 threads an SM
+// again: with one window an SM, its threads are all there is to hide its latencies.
+static uint32_t scan_blocks_resident(uint32_t lambda) {  // blocks an SM holds, of the shape the table picks
     const uint32_t bytes = 4 * window_stride(lambda);
-    uint32_t n = 1;  // blocks an SM holds
-    if (bytes <= 18 * 1024) n = 8;
-    else if (bytes <= 36 * 1024) n = 5;
-    else if (bytes <= 47 * 1024) n = 4;
-    else if (bytes <= 64 * 1024) n = 3;
-    else if (bytes <= 98 * 1024) n = 2;
-    if (blocks <= sms) n = 1;
-    else if (blocks <= 2 * (uint64_t)sms) n = n < 2 ? n : 2;
-    return n == 8 ? 128u : n == 5 ? 224u : n == 4 ? 256u : n == 3 ? 384u : n == 2 ? 512u : 1024u;
+    return bytes <= 18 * 1024 ? 8 : bytes <= 36 * 1024 ? 5 : bytes <= 47 * 1024 ? 4 : bytes <= 64 * 1024 ? 3
+           : bytes <= 98 * 1024 ? 2 : 1;
+}
+
+static uint32_t default_scan_threads(uint32_t lambda, uint64_t blocks, uint32_t sms) {
+    // as many blocks an SM as the launch brings, when that is fewer
+    const uint32_t n = (uint32_t)std::min<uint64_t>(scan_blocks_resident(lambda), (blocks + sms - 1) / sms);
+    return n >= 7 ? 128u : n >= 5 ? 224u : n == 4 ? 256u : n == 3 ? 384u : n == 2 ? 512u : 1024u;
 }
 
 template <int DT, bool QM, int BLOCK>
@@ -2520,10 +2527,19 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
     // the pipelined scan when asked for and its two window arrays fit; any
     // other shape is one block per window (block 0 or 1: the default size)
     const bool pipe = pl.block == SINDI_SCAN_PIPELINED && ix.lambda <= kPipeMaxWindow;
-    const uint32_t block = pl.block > SINDI_SCAN_PIPELINED
-                               ? pl.block
-                               : default_scan_threads(ix.lambda, (uint64_t)nq * ix.sigma * in_flight,
-                                                      (uint32_t)device_sms(ix.device));
+    const uint32_t sms = (uint32_t)device_sms(ix.device);
+    const uint64_t at_once = (uint64_t)nq * in_flight;  // queries the device works on
+    auto block_of = [&](uint32_t windows) {
+        return pl.block > SINDI_SCAN_PIPELINED ? pl.block : default_scan_threads(ix.lambda, at_once * windows, sms);
+    };
+    // A query's first windows run in a launch of their own, and fill its histogram of candidates; the others then
+    // emit only what can still enter the answer (the running bound of Alg. 2's heap, taken from a block of windows
+    // instead of one window at a time). The plain schedule always does; a batch does while its blocks fill the
+    // device but a few times: its windows run in order, but those in flight at once know nothing of each other (one
+    // query over 485 windows: 138 us, now 44).
+    const uint64_t all = at_once * ix.sigma;
+    const bool split = ix.sigma >= kSplitMinWindows &&
+                       (!batched || (all > sms && all < kSplitWaves * (uint64_t)sms * scan_blocks_resident(ix.lambda)));
     const size_t pipe_smem = pipe_smem_bytes(ix.lambda);
     if (batched && !pipe && pl.group > 1 && ix.sigma <= 65535u) {
         // query groups: one block per (group, window); groups vary fastest, so the
@@ -2538,13 +2554,10 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
         const uint64_t items = (uint64_t)nq * ix.sigma;
         const uint32_t blocks = (uint32_t)std::min<uint64_t>(items, (uint64_t)device_sms(ix.device));
         launch_pipe(ix.dtype, sa, blocks, pipe_smem, stream, *chained && !ev0);
-    } else if (!batched && ix.sigma >= kSplitMinWindows) {
-        // One query: its first windows run alone and fill the query's
-        // histogram of candidates; the other windows then emit only what can
-        // still enter the answer (the running bound of Alg. 2's heap, taken
-        // from a block of windows instead of one window at a time).
+    } else if (split) {
         const uint32_t first = std::max<uint32_t>(2u, (ix.sigma + kSplitFraction - 1) / kSplitFraction);
-        launch_scan_pdl(ix.dtype, block, false, sa, first, nq, scan_smem, stream, *chained && !ev0);
+        const bool qm = batched && ix.sigma <= 65535u;
+        launch_scan_pdl(ix.dtype, block_of(first), qm, sa, first, nq, scan_smem, stream, *chained && !ev0);
         ScanArgs sb = sa;
         sb.use_partial = 2;
         sb.w0 = first;
@@ -2554,20 +2567,23 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
             const uint32_t blocks = (sb.nwin + kPlainPipeItems - 1) / kPlainPipeItems;
             launch_pipe(ix.dtype, sb, blocks, pipe_smem, stream, true);
         } else {
-            launch_scan_pdl(ix.dtype, block, false, sb, ix.sigma - first, nq, scan_smem, stream, true);
+            launch_scan_pdl(ix.dtype, block_of(sb.nwin), qm, sb, sb.nwin, nq, scan_smem, stream, true);
         }
         ix.launches += 1;
         ix.scan_launches += 1;
     } else {
         // query-major grids put the queries of one window next to each other
         // (shared lists stay in L2); gridDim.y limits sigma to 65535 there
-        launch_scan_pdl(ix.dtype, block, batched && ix.sigma <= 65535u, sa, ix.sigma, nq, scan_smem,
+        launch_scan_pdl(ix.dtype, block_of(ix.sigma), batched && ix.sigma <= 65535u, sa, ix.sigma, nq, scan_smem,
                         stream, *chained && !ev0);
     }
     if (ev1) SINDI_CUDA(cudaEventRecord(ev1, stream));
     MergeArgs ma{dix, q_indptr, q_indices, q_values, q0, pl.g, pl.final_stage ? 1 : 0, k, out_ids, out_scores, ws};
-    launch_kernel(merge_kernel, dim3(pl.merge_blocks, nq), dim3(kMergeThreads), (size_t)pl.fcap * 8, stream,
-                  !ev1, ma);
+    // two blocks a query: its merge is one block unless its candidates crowd the cut, and every block of the grid is
+    // resident (holding its shared memory) while the scan finishes; a few queries can afford more
+    const uint32_t merge_blocks = std::max<uint32_t>(
+        1, std::min<uint32_t>(pl.cand_cap / 8192, std::max<uint32_t>(2, (uint32_t)(48 / std::min<uint64_t>(at_once, 48)))));
+    launch_kernel(merge_kernel, dim3(merge_blocks, nq), dim3(kMergeThreads), (size_t)pl.fcap * 8, stream, !ev1, ma);
     ix.launches += 2;
     ix.scan_launches += 1;
     if (!pl.final_stage) {
