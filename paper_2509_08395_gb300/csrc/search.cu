@@ -447,8 +447,10 @@ struct TermRed {
     uint32_t m[NW];      // and of max |w_j| (bits of a non-negative float)
     uint32_t q[NW];      // and of the query's largest product bound max_j |w_j| vmax_j, any window
     uint32_t groups[NW]; // posting groups of the warp's terms
+    uint32_t neg[NW];    // 1: one of the warp's terms has a negative query value
     uint32_t total;      // posting groups of the table
     uint32_t qmax;       // the query's largest product bound so far (0 before the first table)
+    uint32_t qneg;       // the query has a negative value so far (0 before the first table; thread 0 writes both)
     int fx_e;            // fixed-point window: its exponent
 };
 
@@ -474,7 +476,7 @@ constexpr uint32_t kPureChunk = 0x8000u;  // c_term: every group of the chunk is
 template <int DT, int BLOCK, bool FX>
 __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w, int32_t j, float qv, int nc, uint4* rec,
                                                   uint32_t* pre, uint16_t* c_term, TermRed<BLOCK / 32>& red,
-                                                  uint32_t* negflag, bool fx_known) {
+                                                  bool fx_known) {
     const DevIndex& ix = a.ix;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nwt = max(1, (nc + 31) >> 5);  // warps with terms
@@ -485,8 +487,8 @@ __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w,
     }
     uint32_t start = 0, len = 0;
     float wq = 0.0f, fb = 0.0f, fm = 0.0f, fq = 0.0f;
+    const bool neg = __any_sync(kFull, tid < nc && qv < 0.0f);
     if (tid < nc) {
-        if (qv < 0.0f) *negflag = 1u;  // a negative query value (any thread may set it)
         if (j >= 0 && j < ix.dim && isfinite(qv) && checked(list_in_bounds(j, w, ix.dim, ix.sigma), ix.err)) {
             const uint64_t sg = (uint64_t)j * ix.sigma + w;
             start = ix.seg[sg];
@@ -522,10 +524,13 @@ __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w,
         }
     }
     const uint32_t q = __reduce_max_sync(kFull, __float_as_uint(fq));
-    if (lane == 0) red.q[warp] = q;
+    if (lane == 0) {
+        red.q[warp] = q;
+        red.neg[warp] = neg ? 1u : 0u;
+    }
     if (lane == 31) red.groups[warp] = incl;
     block_barrier();
-    uint32_t total = 0, M = 0, Q = 0;
+    uint32_t total = 0, M = 0, Q = 0, N = 0;
     float B = 0.0f;
     for (int i = 0; i < nwt; i++) {  // the warps in a fixed order, so that every thread gets the same e
         if (FX && !fx_known) {
@@ -533,6 +538,7 @@ __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w,
             M = max(M, red.m[i]);
         }
         Q = max(Q, red.q[i]);
+        N |= red.neg[i];
         if (i == warp) excl += total;
         total += red.groups[i];
     }
@@ -550,6 +556,7 @@ __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w,
         pre[nc] = total;
         red.total = total;
         red.qmax = max(red.qmax, Q);
+        red.qneg |= N;
         if (FX && !fx_known) red.fx_e = fx_e;
     }
     block_barrier();
@@ -1194,7 +1201,6 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
     __shared__ uint32_t red[kScanWarps + 1];
     __shared__ uint32_t st[4];
     __shared__ uint32_t s_staged;
-    __shared__ uint32_t s_qneg;      // the query has a negative value
     __shared__ uint32_t s_bounded;   // H holds g candidates
     __shared__ SlotBound s_bound;    // and what that means for this window
     __shared__ int32_t s_top;        // H's top bin
@@ -1213,10 +1219,10 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
 
     const int64_t qb = a.q_indptr[r];
     const int nt = (int)(a.q_indptr[r + 1] - qb);
-    if (threadIdx.x == 0) {  // read after the term tables' barriers
-        s_qneg = 0;
+    if (threadIdx.x == 0) {  // read after the term tables' barriers, and until then written by this thread only
         s_staged = 0;
-        tred.qmax = 0;  // (written again only by this thread)
+        tred.qmax = 0;
+        tred.qneg = 0;
     }
     // the window is zeroed in two halves, while the query's offsets and then its terms are on their way
     float4* A4 = reinterpret_cast<float4*>(A);
@@ -1250,7 +1256,7 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
         }
         s_bounded = found ? 1u : 0u;
         // zero-score slots cannot count once the earlier windows hold g slots, when no score can be negative
-        const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
+        const bool skip_zero = tred.qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
         if (found) s_bound = slot_bound(bin, top, skip_zero, FX ? tred.fx_e : kNoFx);
     };
 
@@ -1267,7 +1273,7 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
             }
             __syncthreads();  // previous table fully consumed
         }
-        build_group_table<DT, BLOCK, FX>(a, w, j, qv, nc, t_rec, t_pre, c_term, tred, &s_qneg, fx_pre);
+        build_group_table<DT, BLOCK, FX>(a, w, j, qv, nc, t_rec, t_pre, c_term, tred, fx_pre);
         if (a.use_partial != 2 && warp == kBoundWarp && c0 + kTermChunk >= nt) publish_bound();
         accumulate_groups<DT, kScanWarps, FX>(ix, t_rec, t_pre, c_term, nc, tred.total, warp, lane, A);
     }
@@ -1289,7 +1295,7 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
     if (!direct) {
         const int64_t rest = ix.n_docs - (int64_t)w * lambda;
         const int n_eff = (int)(rest < (int64_t)lambda ? rest : (int64_t)lambda);
-        const bool skip_zero = s_qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
+        const bool skip_zero = tred.qneg == 0 && ix.nonneg && (uint64_t)w * lambda >= a.g;
         if ((uint32_t)n_eff <= a.win_cap) {
             // the window's budget holds all its slots (a deep pool over a small window): no cut to look for
             if (threadIdx.x == 0) {
