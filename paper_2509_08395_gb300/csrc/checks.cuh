@@ -41,6 +41,14 @@ SINDI_HD bool list_in_bounds(int32_t j, uint32_t w, int32_t dim, uint32_t sigma)
     return j >= 0 && j < dim && w < sigma;
 }
 
+// Terms c0 .. of a query row of nt entries that a table of `block` terms takes.
+// A row whose device offsets decrease (nt < 0: only host offsets are checked
+// before a search) has none, so that nothing is indexed by a negative count.
+SINDI_HD int table_terms(int nt, int c0, int block) {
+    const int rest = nt > c0 ? nt - c0 : 0;
+    return rest < block ? rest : block;
+}
+
 // A document id (candidate or result) of an index of n documents.
 SINDI_HD bool doc_in_bounds(uint32_t id, int64_t n) { return (int64_t)id < n; }
 

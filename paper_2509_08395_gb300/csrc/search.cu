@@ -1265,7 +1265,7 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
     const bool fx_pre = FX && nt > kTermChunk;
     if (fx_pre) window_scale_exp<DT, BLOCK>(a, w, qb, nt, tred, reinterpret_cast<float*>(region));
     for (int c0 = 0; c0 == 0 || c0 < nt; c0 += kTermChunk) {
-        const int nc = min(kTermChunk, nt - c0);
+        const int nc = table_terms(nt, c0, kTermChunk);  // (the first table is built for an empty query too)
         if (c0) {
             if ((int)threadIdx.x < nc) {
                 j = a.q_indices[qb + c0 + threadIdx.x];
