@@ -850,9 +850,11 @@ __device__ __forceinline__ void sample_cut(const float* A, int n_eff, uint32_t g
         }
 #pragma unroll
         for (int c = 0; c < 4; c++) {
-            // (slots past n_eff were never added to: 0, which is in no bin but the lowest unless all scores are)
-            const uint32_t bin = hbin(float_order_bits(v[c]), top);
-            if (bin && 4 * i4 + c < n_eff) atomicAdd(&hist[bin], 1u);
+            // (most slots hold 0: not counted, nor are scores next to it)
+            if (v[c] > 0.0f) {
+                const uint32_t bin = hbin(float_order_bits(v[c]), top);
+                if (bin > (uint32_t)kHRest && 4 * i4 + c < n_eff) atomicAdd(&hist[bin], 1u);
+            }
         }
     }
     __syncthreads();
@@ -1248,7 +1250,7 @@ __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_
     // what the bin means for this window (after the last term table's barriers)
     auto publish_bound = [&]() {
         if (lane != 0) return;
-        const int32_t top = hbin_top(float_order_bits(__uint_as_float(tred.qmax)));
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(tred.qmax)), nt);
         s_top = top;
         if (w == 0) {
             wait_previous_kernels();
@@ -1457,7 +1459,8 @@ __global__ void __launch_bounds__(kPipeThreads, 1) scan_pipe_kernel(ScanArgs a) 
         if (it == 0) wait_previous_kernels();
         if (it + 1 == n_my) allow_next_kernel();
         // the query's running bound: g candidates emitted at or above a bin
-        const int32_t top = hbin_top(float_order_bits(__uint_as_float(qmax)));
+        const int64_t qr = a.q_first + y;
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(qmax)), (int)(a.q_indptr[qr + 1] - a.q_indptr[qr]));
         if (S::tid() < 32) {
             uint32_t hb = 0;
             const bool f = warp_find_bound(a.ws.hist + (size_t)y * kHBins, a.g, &hb);
@@ -1718,7 +1721,7 @@ __global__ void __launch_bounds__(BLOCK, 1024 / BLOCK) group_scan_kernel(GroupSc
         const uint32_t y = mrow[i];
         // the query's running bound: g candidates emitted at or above some bin (H only
         // grows while the launch runs, so any read of it bounds the answer)
-        const int32_t top = hbin_top(float_order_bits(__uint_as_float(s_qmax[i])));
+        const int32_t top = hbin_top(float_order_bits(__uint_as_float(s_qmax[i])), (int)(mpre[i + 1] - mpre[i]));
         if (warp == 0) {
             uint32_t hb = 0;
             const bool f = warp_find_bound(sa.ws.hist + (size_t)y * kHBins, sa.g, &hb);
