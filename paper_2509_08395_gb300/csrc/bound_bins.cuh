@@ -34,8 +34,12 @@ constexpr int kHRest = kHBins - 1 - (kHFine + kHMid + kHLow);  // other scores >
 
 // The top bin's place, from the order bits (float_order_bits) of M and the query's number of terms.
 SINDI_HD int32_t hbin_top(uint32_t order_bits, int terms = 8) {
+#ifdef __CUDA_ARCH__
+    const int octaves = terms > 8 ? 32 - __clz(terms - 1) : 3;
+#else
     int octaves = 3;
-    while (octaves < 30 && terms > 1 << octaves) octaves++;
+    while (octaves < 31 && (int64_t)terms > (int64_t)1 << octaves) octaves++;
+#endif
     return (int32_t)(order_bits >> 17) + octaves * 64;
 }
 
