@@ -459,6 +459,12 @@ __device__ __forceinline__ void block_barrier() { asm volatile("barrier.cta.sync
 
 constexpr uint32_t kPureChunk = 0x8000u;  // c_term: every group of the chunk is one term's, whole
 
+// kPureChunk when chunk c lies in the whole groups of a term: groups excl .. next - 1 of the table, postings start .. end - 1.
+__device__ __forceinline__ uint32_t pure_chunk(uint32_t c, uint32_t excl, uint32_t next, uint32_t start, uint32_t end) {
+    const uint32_t whole0 = excl + ((start & 7u) ? 1u : 0u), whole1 = next - ((end & 7u) ? 1u : 0u);
+    return 32u * c >= whole0 && 32u * c + 32u <= whole1 ? kPureChunk : 0u;
+}
+
 // The term table of one query over one window for the window scan, for terms c0 .. c0 + nc - 1 of the query (nc <=
 // BLOCK, one term a thread). A term's segment is tiled on 8-aligned groups of 8 postings; the groups of all terms,
 // in term order, are numbered through, and a warp chunk is 32 consecutive groups, one a lane, whatever terms they
@@ -547,10 +553,8 @@ __device__ __forceinline__ void build_group_table(const ScanArgs& a, uint32_t w,
         const float wr = FX ? wq * pow2f(fx_e) : wq;  // exact (the exponent's clamps)
         rec[tid] = make_uint4((start & ~7u) - 8u * excl, start, end, __float_as_uint(wr));
         pre[tid] = excl;
-        const uint32_t whole0 = excl + ((start & 7u) ? 1u : 0u), whole1 = excl + ng - ((end & 7u) ? 1u : 0u);
         for (uint32_t c = (excl + 31u) >> 5; 32u * c < excl + ng && c < (uint32_t)kChunkTable; c++)
-            c_term[c] = (uint16_t)((uint32_t)tid |
-                                   (32u * c >= whole0 && 32u * c + 32u <= whole1 ? kPureChunk : 0u));
+            c_term[c] = (uint16_t)((uint32_t)tid | pure_chunk(c, excl, excl + ng, start, end));
     }
     if (tid == 0) {
         pre[nc] = total;
@@ -577,7 +581,14 @@ __device__ __forceinline__ void load_group(const DevIndex& ix, const uint4* rec,
                                            const uint16_t* c_term, int nc, uint32_t total, uint32_t c, int lane,
                                            Group8& k) {
     const uint32_t G = 32u * c + (uint32_t)lane;
-    const uint32_t ct = c < (uint32_t)kChunkTable ? (uint32_t)c_term[c] : (uint32_t)term_of(pre, nc, 32u * c);
+    uint32_t ct;
+    if (c < (uint32_t)kChunkTable) {
+        ct = (uint32_t)c_term[c];
+    } else {
+        // past the table: windows of thousands of chunks (dense documents), nearly all of one term each
+        ct = (uint32_t)term_of(pre, nc, 32u * c);
+        ct |= pure_chunk(c, pre[ct], pre[ct + 1], rec[ct].y, rec[ct].z);
+    }
     k.lm = 0xFFu;
     if (ct & kPureChunk) {
         // about 7 in 10 chunks of the 1M-document workload
