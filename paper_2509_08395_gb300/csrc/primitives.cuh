@@ -8,6 +8,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace sindi {
@@ -26,6 +28,18 @@ struct Pool {
         size_t bytes = count * sizeof(T);
         if (bytes == 0) bytes = 16;
         SINDI_CUDA(cudaMallocFromPoolAsync(&p, bytes, pool, stream));
+        return static_cast<T*>(p);
+    }
+    // nullptr when the device has no room for it
+    template <typename T>
+    T* try_alloc(size_t count) {
+        void* p = nullptr;
+        const cudaError_t e = cudaMallocFromPoolAsync(&p, std::max<size_t>(count * sizeof(T), 16), pool, stream);
+        if (e == cudaErrorMemoryAllocation) {
+            (void)cudaGetLastError();
+            return nullptr;
+        }
+        SINDI_CUDA(e);
         return static_cast<T*>(p);
     }
     void free(void* p) {

@@ -40,6 +40,7 @@
 #include "common.cuh"
 #include "fixed_point.cuh"
 #include "index.cuh"
+#include "launch_rules.cuh"
 #include "mass.cuh"
 #include "primitives.cuh"
 
@@ -2761,8 +2762,8 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
     const bool batched = prm.mode == SINDI_MODE_BATCHED;
     int64_t chunk = 1;
     if (batched) {
-        // workspace per launch group: every group reads the lists again and ends in a wave that is not full (1,000
-        // queries over 8.8M documents: 2 GiB 18.85 ms, 4 GiB 18.39)
+        // workspace per launch group, if there is room for it: every group reads the lists again and ends in a wave
+        // that is not full (1,000 queries over 8.8M documents: 2 GiB 18.85 ms, 4 GiB 18.39)
         const size_t budget = (size_t)4 << 30;
         const size_t per_query = workspace_bytes(1, pl.cand_cap, pl.fcap, pl.top_cap);
         chunk = std::max<int64_t>(1, std::min<int64_t>(n_queries, (int64_t)(budget / per_query)));
@@ -2815,15 +2816,6 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
         ix.graph_seen = failed ? IndexImpl::PlainCall{} : call;
     }
     Pool P{ix.pool, stream};
-    const size_t ws_one = workspace_bytes(chunk, pl.cand_cap, pl.fcap, pl.top_cap);
-    const size_t ws_stride = (ws_one + 255) & ~(size_t)255;
-    unsigned char* mem = P.alloc<unsigned char>(ws_stride * lanes);
-    std::vector<Workspace> wss;
-    for (int l = 0; l < lanes; l++) {
-        wss.push_back(carve_workspace(mem + ws_stride * l, chunk, pl.cand_cap, pl.fcap, pl.top_cap));
-        SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_clear_bytes(chunk), stream));
-    }
-    const Workspace& ws = wss[0];
     QueryCsr pruned{nullptr, nullptr, nullptr};
     int64_t* pq_indptr = nullptr;
     int32_t* pq_idx = nullptr;
@@ -2856,6 +2848,29 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
         ix.launches += 3;
         pruned = QueryCsr{pq_indptr, pq_idx, pq_val};
     }
+    auto free_pruned = [&]() {
+        for (void* p : {(void*)pq_kept, (void*)tq_idx, (void*)tq_val, (void*)pq_indptr, (void*)pq_idx, (void*)pq_val})
+            P.free(p);
+    };
+    unsigned char* mem = nullptr;
+    size_t ws_stride = 0;
+    auto get_workspaces = [&](int64_t c) {
+        ws_stride = align256(workspace_bytes(c, pl.cand_cap, pl.fcap, pl.top_cap));
+        mem = P.try_alloc<unsigned char>(ws_stride * lanes);
+        return mem != nullptr;
+    };
+    // last of the call's allocations: a batch takes smaller groups where the device has no room for the full one
+    chunk = largest_that_fits(chunk, get_workspaces);
+    if (chunk == 0) {
+        free_pruned();
+        throw CudaError{cudaErrorMemoryAllocation, "the search's workspace"};
+    }
+    std::vector<Workspace> wss;
+    for (int l = 0; l < lanes; l++) {
+        wss.push_back(carve_workspace(mem + ws_stride * l, chunk, pl.cand_cap, pl.fcap, pl.top_cap));
+        SINDI_CUDA(cudaMemsetAsync(mem + ws_stride * l, 0, workspace_clear_bytes(chunk), stream));
+    }
+    const Workspace& ws = wss[0];
 
     std::vector<cudaEvent_t> evs;
     bool chained = false;
@@ -2889,12 +2904,7 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
     }
     ix.queries += (uint64_t)n_queries;
     P.free(mem);
-    P.free(pq_kept);
-    P.free(tq_idx);
-    P.free(tq_val);
-    P.free(pq_indptr);
-    P.free(pq_idx);
-    P.free(pq_val);
+    free_pruned();
     if (timing) {
         SINDI_CUDA(cudaStreamSynchronize(stream));
         double ms = 0.0;
