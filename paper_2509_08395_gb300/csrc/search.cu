@@ -46,11 +46,9 @@
 
 namespace sindi {
 
-constexpr int kPlainLanes = 24;            // plain schedule: query chains in flight at once, launched one by one
-constexpr int kGraphLanes = 56;            // and in a recorded graph, at most (graph_lanes)
 constexpr uint32_t kPlainPipeItems = 6;    // plain schedule, pipelined scan: windows per block
-constexpr uint32_t kSplitMinWindows = 8;   // plain schedule: a query of this many windows or more scans
-constexpr uint32_t kSplitFraction = 8;     // its first 1/kSplitFraction windows first; a batch does the same while
+constexpr uint32_t kSplitFraction = 8;     // plain schedule: a query of kSplitMinWindows windows or more scans its
+                                           // first 1/kSplitFraction windows first; a batch does the same while
 constexpr uint64_t kSplitWaves = 6;        // its blocks fill the device fewer times than this
 constexpr int kMaxScanWarps = 1024 / 32;   // largest scan block
 constexpr int kChunkTable = 1024;          // chunks mapped to their list by a table (then a search)
@@ -2629,21 +2627,6 @@ static void launch_group(const IndexImpl& ix, const Plan& pl, const Workspace& w
     *chained = true;
 }
 
-// Chains in flight of the plain schedule's recorded graph. A chain is a few microseconds of scan on many SMs and then
-// latency on few, so a long call gains from more of them than the host can feed launch by launch; measured, ms a
-// call of 1,000 queries (300 in the last row):
-//   chains                       24    40    56    64
-//   1M documents, 62 windows   2.89  2.76  2.74  2.75
-//   300k, 37 windows           2.07  1.47  1.36  1.37
-//   200k, 13 windows           1.96  1.34  1.11  1.10
-//   400k, 25 windows           0.70  0.56  0.56  0.55
-// A chain holds several queries, and an index of a few windows keeps 24 (100 exact queries over three windows: 24
-// chains 109 us, 32 120, 40 122).
-static int graph_lanes(const IndexImpl& ix, int64_t n_queries) {
-    if (ix.sigma < kSplitMinWindows) return kPlainLanes;
-    return (int)std::max<int64_t>(kPlainLanes, std::min<int64_t>(kGraphLanes, n_queries / 5));
-}
-
 // The plain schedule's launches: query i's chain on lane i mod lanes. Every
 // lane starts after the work already on `stream` (fork event) and `stream`
 // continues after every lane (join events). The events go to `evs`; the
@@ -2797,12 +2780,18 @@ sindi_status search_impl(const IndexImpl& ix, const int64_t* q_indptr, const int
         std::lock_guard<std::mutex> lk(ix.graph_mu);
         bool failed = false;
         if (!(ix.graph_exec && ix.graph_call == call) && ix.graph_seen == call) {
-            try {
-                capture_plain_graph(ix, pl, call, (int)std::min<int64_t>(graph_lanes(ix, n_queries), n_queries),
-                                    q_indptr, q_indices, q_values, n_queries, k, out_ids, out_scores);
-            } catch (const CudaError&) {
-                (void)cudaGetLastError();
-                failed = true;  // launch directly, and do not try this call again
+            // where the device has no room for that many chains' workspaces, for as many as direct launches use
+            const int many = graph_lanes(ix.sigma, n_queries, workspace_bytes(1, pl.cand_cap, pl.fcap, pl.top_cap));
+            for (int n : {many, lanes}) {
+                try {
+                    capture_plain_graph(ix, pl, call, n, q_indptr, q_indices, q_values, n_queries, k, out_ids,
+                                        out_scores);
+                } catch (const CudaError& e) {
+                    (void)cudaGetLastError();
+                    if (e.code == cudaErrorMemoryAllocation && n > lanes) continue;
+                    failed = true;  // launch directly, and do not try this call again
+                }
+                break;
             }
         }
         if (ix.graph_exec && ix.graph_call == call) {

@@ -19,6 +19,8 @@ int main(int argc, char** argv) {
         long long tries = 0;
         const long long got = largest_that_fits(a, [&](int64_t c) { tries++; return c <= b; });
         std::printf("%lld %lld\n", got, tries);
+    } else {  // a windows, b queries, bytes a chain
+        std::printf("%d 0\n", graph_lanes((uint32_t)a, b, (size_t)std::atoll(argv[4])));
     }
     return 0;
 }
@@ -45,3 +47,20 @@ def test_a_batch_takes_the_largest_group_there_is_room_for(run, n):
             assert (got, tries) == (n, 1)
         else:  # a group of more than half of what fits, and never less than one query
             assert 1 <= got <= room and 2 * got >= room
+
+
+MIB = 1 << 20
+
+
+@pytest.mark.parametrize("sigma", [1, 7, 8, 62, 1075])
+@pytest.mark.parametrize("queries", [2, 23, 100, 119, 120, 200, 1000, 100_000])
+@pytest.mark.parametrize("lane_bytes", [100_000, 512 * 1024, 17 * MIB, 21 * MIB, 22 * MIB, 141 * MIB, 4096 * MIB])
+def test_more_chains_only_while_their_workspaces_are_small(run, sigma, queries, lane_bytes):
+    lanes, _ = run("lanes", sigma, queries, lane_bytes)
+    assert 1 <= lanes <= min(56, queries)
+    assert lanes >= min(24, queries)  # what direct launches use
+    assert lanes <= 24 or lanes * lane_bytes <= 512 * MIB
+    if sigma < 8 or queries <= 120 or lane_bytes >= 22 * MIB:
+        assert lanes == min(24, queries)
+    if sigma >= 8 and queries >= 280 and lane_bytes <= 9 * MIB:
+        assert lanes == 56
