@@ -244,7 +244,8 @@ sindi_status sindi_build(const int64_t* indptr, const int32_t* indices, const fl
  * buffers, n_queries, k, gamma and block shape; beta = 1; timing off; stream
  * not being captured) comes a second time, its launches are recorded as one
  * CUDA graph with working memory of its own (held until the index is freed
- * or another call is recorded); identical calls then launch the graph, which
+ * or another call is recorded: a workspace for each of 24 chains, or for up
+ * to 56 while all of them take at most 512 MiB); identical calls then launch the graph, which
  * reads the buffers' current contents. A plain call on a stream that is not
  * being captured first waits (on the GPU) for the graph's previous launch, so
  * launches from different streams never share its working memory at once.
@@ -439,6 +440,19 @@ sindi_status sindi_index_export(const sindi_index* index, uint32_t* seg, uint16_
 sindi_status sindi_set_timing(const sindi_index* index, int enable);
 sindi_status sindi_get_stats(const sindi_index* index, sindi_stats_t* out);
 sindi_status sindi_reset_stats(const sindi_index* index);
+
+/*
+ * Return to the system the device memory that the library holds on `device`
+ * without using it. The library allocates from a memory pool of its own and
+ * keeps what it frees for the next call: the memory of freed indexes (until
+ * the next build), the workspaces of searches (a batch's at most 4 GiB, or
+ * what one query needs), and up to 1 GiB of a build's temporaries. Other allocators of the process
+ * cannot use that memory until it is returned here. Memory in use, also by
+ * work that is still queued, stays. May be called from any thread at any
+ * time; the next build or search allocates anew. SINDI_ERR_INVALID_ARG for a
+ * device that does not exist.
+ */
+sindi_status sindi_release_memory(int32_t device);
 
 /* Free an index and everything it owns. NULL is ignored. Waits for work
    queued on the index's streams to finish. Plans and servers over the index

@@ -32,12 +32,13 @@ bool trace_on() {
 }
 
 // One pool per device, owned by the library, that keeps freed blocks for
-// reuse (release threshold = unlimited); big temporaries of a build are
-// returned with an explicit trim.
+// reuse (release threshold = unlimited). A build returns its temporaries but
+// for a reserve (trim_pool); sindi_release_memory returns all that is unused.
+static std::mutex pools_mu;
+static std::map<int, cudaMemPool_t> pools;
+
 cudaMemPool_t library_pool(int device) {
-    static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
-    std::lock_guard<std::mutex> lk(mu);
+    std::lock_guard<std::mutex> lk(pools_mu);
     auto it = pools.find(device);
     if (it != pools.end()) return it->second;
     cudaMemPoolProps props = {};
@@ -53,7 +54,8 @@ cudaMemPool_t library_pool(int device) {
 }
 
 // Returns a build's temporaries to the system, all but kPoolReserve bytes beyond what is in use: mapping and unmapping
-// them took 1 of the 4 ms an index of 1M documents is built in when indexes are built one after another.
+// them took 1 of the 4 ms an index of 1M documents is built in when indexes are built one after another. (What is kept,
+// and what a freed index or a search leaves, other allocators of the process cannot use: sindi_release_memory.)
 constexpr uint64_t kPoolReserve = (uint64_t)1 << 30;
 static void trim_pool(cudaMemPool_t pool) {
     uint64_t used = 0;
@@ -832,6 +834,32 @@ void sindi_index_free(sindi_index* index) {
         free_index_memory(index->impl, nullptr);
     }
     delete index;
+}
+
+sindi_status sindi_release_memory(int32_t device) {
+    set_last_error("");
+    int devices = 0;
+    if (cudaGetDeviceCount(&devices) != cudaSuccess) {
+        (void)cudaGetLastError();
+        devices = 0;
+    }
+    if (device < 0 || device >= devices) {
+        set_last_error("no such device");
+        return SINDI_ERR_INVALID_ARG;
+    }
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(pools_mu);
+        auto it = pools.find(device);
+        if (it == pools.end()) return SINDI_OK;  // nothing was ever allocated there
+        pool = it->second;
+    }
+    try {
+        SINDI_CUDA(cudaMemPoolTrimTo(pool, 0));
+    } catch (const CudaError& e) {
+        return from_cuda(e);
+    }
+    return SINDI_OK;
 }
 
 }  // extern "C"

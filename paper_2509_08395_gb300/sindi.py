@@ -108,6 +108,7 @@ _SIGS = {
     "sindi_get_stats": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(sindi_stats_t)]),
     "sindi_reset_stats": (ctypes.c_int, [ctypes.c_void_p]),
     "sindi_index_free": (None, [ctypes.c_void_p]),
+    "sindi_release_memory": (ctypes.c_int, [ctypes.c_int32]),
     "sindi_plan_create": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                          ctypes.c_int64, ctypes.POINTER(sindi_search_params), ctypes.c_void_p,
                                          ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p)]),
@@ -306,6 +307,12 @@ def sindi_reset_stats(index: int) -> None:
 def sindi_index_free(index: int) -> None:
     if index:
         load().sindi_index_free(ctypes.c_void_p(index))
+
+
+def sindi_release_memory(device: int = 0) -> None:
+    """Returns the device memory the library keeps without using it (freed indexes, search workspaces, up to 1 GiB of
+    a build's temporaries), so that other allocators can have it."""
+    _check(load().sindi_release_memory(int(device)), "sindi_release_memory")
 
 
 def sindi_version() -> str:
