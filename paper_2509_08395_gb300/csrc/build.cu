@@ -57,6 +57,7 @@ struct PruneArgs {
     uint32_t* n_sort;
     uint32_t* long_rows;   // rows left to prune_long_rows_kernel, and their count
     uint32_t* n_long;
+    uint32_t* next_long;   // rows of that list that a block has taken
     uint32_t* err;
 };
 
@@ -362,20 +363,26 @@ __global__ void __launch_bounds__(kPruneWarps * 32) prune_rows_kernel(PruneArgs 
     }
 }
 
-// One block per listed long row (kPruneRowCap < m <= kMaxRowNnz); same rules.
+// One block per listed long row (kPruneRowCap < m <= kMaxRowNnz); same rules. A block takes the next row when it is done
+// with one: rows of 2,000 to 6,000 entries differ by four in their sorts, and shared out beforehand they left SMs idle.
 constexpr int kLongBlock = 512;
 __global__ void __launch_bounds__(kLongBlock) prune_long_rows_kernel(PruneArgs p) {
     extern __shared__ uint64_t s[];
     __shared__ int flags[2];
     __shared__ int s_r, s_nz;
+    __shared__ uint32_t s_row;
     const uint32_t n_rows = *p.n_long;
-    for (uint32_t row = blockIdx.x; row < n_rows; row += gridDim.x) {
+    while (true) {
+        __syncthreads();  // the previous row is done with the shared arrays
+        if (threadIdx.x == 0) s_row = atomicAdd(p.next_long, 1u);
+        __syncthreads();
+        const uint32_t row = s_row;
+        if (row >= n_rows) break;
         const int64_t i = p.long_rows[row];
         const int64_t b = p.indptr[i];
         const int mm = (int)(p.indptr[i + 1] - b);
         int p2 = 32;
         while (p2 < mm) p2 <<= 1;
-        __syncthreads();  // the previous row is done with the shared arrays
         if (threadIdx.x == 0) { flags[0] = 0; flags[1] = 0; s_nz = 0; }
         __syncthreads();
         for (int t = threadIdx.x; t < p2; t += kLongBlock) {
@@ -807,14 +814,15 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
     uint32_t* kept = ix.kept;
     const size_t mask_words = (size_t)keep_words(nnz, n) + 1;
     uint32_t* mask = P.alloc<uint32_t>(mask_words);
-    uint32_t* left_rows = P.alloc<uint32_t>(2 * (size_t)n + 2);  // rows to sort, long rows, their counts
+    uint32_t* left_rows = P.alloc<uint32_t>(2 * (size_t)n + 3);  // rows to sort, long rows, their counts, rows taken
     uint32_t* n_left = left_rows + 2 * n;
-    SINDI_CUDA(cudaMemsetAsync(n_left, 0, 8, stream));
+    SINDI_CUDA(cudaMemsetAsync(n_left, 0, 12, stream));
     SINDI_TRACE_MSG("build_lists: launching the pruning kernels");
     int64_t* kept_off = P.alloc<int64_t>(n + 1);
     if (n > 0) {
         const PruneArgs pa{ix.indptr, ix.indices, ix.values, n,         d,          ix.alpha,      vn,
-                           kept,      mask,       left_rows, n_left,    left_rows + n, n_left + 1, ix.err};
+                           kept,      mask,       left_rows, n_left,    left_rows + n, n_left + 1, n_left + 2,
+                           ix.err};
         // rows per warp: as many as leave four waves of warps
         const int rows = (int)std::min<int64_t>(32, std::max<int64_t>(1, n / (152 * 32 * 4)));
         const unsigned blocks = (unsigned)((n + (int64_t)rows * kSelectWarps - 1) / ((int64_t)rows * kSelectWarps));
