@@ -930,12 +930,12 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         // When the slots that can count fit the window's budget, emit all of them:
         // no window histogram, no cut. One pass stages them (a shared counter: a
         // few dozen a bounded window), then one reservation for the group. Under a
-        // loose bound (ties) thousands may count: a thread that finds the budget
-        // passed stops, and the cut below reads the window anew (100 queries of one
-        // term over 1M documents, a quarter of them tied at the top: 1.96 -> 1.87 ms
-        // one by one, 1.64 -> 1.55 batched; the look at the counter costs 0.8% of a
-        // batch over lognormal documents, and every other form tried cost more:
-        // one add per warp 3.5%, a flag 1.2%, giving up on the add's own result 9%).
+        // loose bound (ties) thousands may count, and are staged before the cut below
+        // reads the window anew: stopping once the budget is passed was measured, and
+        // gave 5% there (100 queries of one term, a quarter of 1M documents tied: 1.64
+        // -> 1.55 ms a batch) but cost 0.7 to 1.2% of every ordinary search in its
+        // cheapest form (a look at the counter: 1,000 queries over 1M lognormal
+        // documents 2.119 -> 2.135 ms), and places taken by one add per warp 3.5%.
         const float thr = b.thr;
         const int n4 = (n_eff + 3) >> 2;
         const float4* A4 = reinterpret_cast<const float4*>(A);
@@ -943,7 +943,6 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
         const int32_t ithr = b.ithr;
         // the window 4 slots per lane and load, four loads in flight; the per-slot work runs only for the
         // rare lane that holds a candidate
-        auto passed = [&]() { return *static_cast<volatile uint32_t*>(cs.s_staged) > a.win_cap; };
         auto scan_bounded = [&](auto&& emit) {
             if (fx) {
                 auto look = [&](const int4& x, int i) {
@@ -962,7 +961,6 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
                     m = max(m, max(max(x2.x, x2.y), max(x2.z, x2.w)));
                     m = max(m, max(max(x3.x, x3.y), max(x3.z, x3.w)));
                     if (m >= ithr) {
-                        if (passed()) return;
                         look(x, 4 * i4);
                         look(x1, 4 * (i4 + NT));
                         look(x2, 4 * (i4 + 2 * NT));
@@ -975,7 +973,6 @@ __device__ void select_window(const ScanArgs& a, float* A, uint32_t w, uint32_t 
                 for (int i4 = tid; i4 < n4; i4 += NT) {
                     const float4 x = A4[i4];
                     if (x.x >= thr || x.y >= thr || x.z >= thr || x.w >= thr) {
-                        if (passed()) return;
                         const int i = 4 * i4;
                         if (x.x >= thr) emit(i);
                         if (x.y >= thr && i + 1 < n_eff) emit(i + 1);
