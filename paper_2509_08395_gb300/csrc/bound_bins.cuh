@@ -16,7 +16,7 @@
 // over data of many similar products, as uniform or binary vectors have, lay in
 // the top bin, and with one bin for zero and all negative scores answers below
 // zero had no bound: 200 queries of 20 terms over 1M binary documents of 60
-// entries, 500 candidates, took 3.52 ms one by one and 1.93 batched, now 1.71 and
+// entries, 500 candidates, took 3.52 ms one by one and 1.93 batched, now 1.70 and
 // 0.91; with 8 bins an octave everywhere 2.04 and 1.37.)
 #pragma once
 

@@ -138,11 +138,14 @@ struct CudaError {
 
 inline uint32_t ceil_div_u32(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
-// How the window scan reads a list segment I_{j,w}, which the build's posting
-// order follows: a warp chunk is 256 postings of one segment; a segment of at
-// least kVecMin postings is tiled on 8-aligned groups (lane l of a chunk owns
-// the l-th group of 8, one posting per add instruction u = 0..7); a shorter
-// segment is one chunk whose lane l owns postings s + l + 32u.
+// The chunks of a list segment I_{j,w} that the build's posting order is laid
+// out for, and that the pipelined and query-group scans read: a warp chunk is
+// 256 postings of one segment; a segment of at least kVecMin postings is tiled
+// on 8-aligned groups (lane l of a chunk owns the l-th group of 8, one posting
+// per add instruction u = 0..7); a shorter segment is one chunk whose lane l
+// owns postings s + l + 32u. The default scan numbers the 8-aligned groups of
+// all terms through and takes 32 consecutive ones, so its chunks begin anywhere
+// in a segment and may cross into the next term's.
 constexpr int kChunkU = 8;                 // postings per lane in one warp chunk
 constexpr int kChunkLen = 32 * kChunkU;    // postings of one warp chunk (one list only)
 constexpr uint32_t kVecMin = 32;           // segments this long are read with vector loads

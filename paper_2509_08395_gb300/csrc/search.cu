@@ -6,26 +6,29 @@
 //       A[lambda] in shared memory (Alg. 2, the product + accumulation loops):
 //       FP32 sums, or 32-bit fixed-point sums of the FP32 products (the default
 //       when the search reorders; fixed_point.cuh), read as FP32 scores by the
-//       cut. The block then histograms the window's scores on the top 12
-//       bits of their order key and emits every slot in the bins at or above
-//       the bin that holds its g-th best slot (the window's share of the heap
-//       update of Alg. 2). When ties crowd that bin, an exact radix select
-//       emits exactly the best g. Each block adds the histogram of what it
-//       emitted to a per-query histogram H. Where earlier windows of the query
-//       are complete (batched schedules: a snapshot taken at the block's
-//       start; the plain schedule's second launch: H read after the
-//       accumulation), a bin reached by g already emitted slots bounds what
-//       can still enter the answer, and a window whose slots above that bound
-//       fit its budget emits them in one pass, with no cut.
+//       cut. Each block counts what it emits in a per-query histogram H
+//       (bound_bins.cuh). Where earlier windows of the query are complete
+//       (batched schedules: a snapshot taken at the block's start; a second
+//       launch over a query's later windows: H read after the accumulation),
+//       a bin reached by g already emitted slots bounds what can still enter
+//       the answer, and a window whose slots above that bound fit its budget
+//       of 2 g emits them in one pass, with no cut (the window's share of the
+//       heap update of Alg. 2). A window without a bound guesses one from a
+//       sample of its slots (sample_cut) and goes the same way when between g
+//       and 2 g slots reach it. Otherwise the full cut decides: the scores are
+//       histogrammed on the top 12 bits of their order key in the 256 bins from
+//       the window's best down, then on 8 more bits inside the bin of the g-th
+//       best, and an exact radix select emits the best g when ties crowd the
+//       cut or it lies below those bins.
 //   merge        (one block per query up to 16384 candidates, a few above):
 //       from H, the bin of the global g-th best candidate; candidates below
 //       it are dropped, the rest (about g) gathered and the exact best g
 //       selected in shared memory (the heap H of Alg. 2 across windows).
 //       With gamma = 0 these are the sorted results; otherwise they are the
 //       gamma reorder candidates.
-//   rerank       (one half-warp per candidate): delta(x_i, q) from the
-//       unpruned document and the unpruned query (Alg. 4, the reorder loop);
-//       the last block of a query sorts the scores and writes the top k.
+//   rerank       (a half-warp scores 1 to 16 candidates in turn): delta(x_i, q)
+//       from the unpruned document and the unpruned query (Alg. 4, the reorder
+//       loop); the last block of a query sorts the scores and writes the top k.
 //
 // Order keys (common.cuh) make every comparison exact: (score desc, id asc).
 #include <cuda_fp16.h>
@@ -1201,8 +1204,8 @@ constexpr int scan_blocks_per_sm(int block) { return block == 384 ? 3 : block ==
 // from L2), and the barriers between its phases. With chunks of one term each,
 // a 12-bit H read by all threads, a barrier per table step and 37 KiB of
 // scratch beside every window (two blocks an SM at best), 1,000 queries over
-// 1M documents (16,384-slot windows) took 3.59 ms a batch, now 2.34; over 8.8M
-// (8,192 slots, FP16) 40.2, now 19.3; exact search of uniform vectors (segments
+// 1M documents (16,384-slot windows) took 3.58 ms a batch, now 2.12; over 8.8M
+// (8,192 slots, FP16) 39.9, now 17.1; exact search of uniform vectors (segments
 // of 64 postings) 0.69, now 0.34.
 template <int DT, bool QUERY_MAJOR, int BLOCK, bool FX>
 __global__ void __launch_bounds__(BLOCK, scan_blocks_per_sm(BLOCK)) scan_window_kernel(ScanArgs a) {
@@ -2134,7 +2137,7 @@ static size_t rerank_dyn_bytes(uint32_t top_cap) {
 // the time of the 16 rows its half-warps hold, so a large batch gives each half-warp up to 16 rounds, whose keys and
 // row offsets are read at once (lane l: round l). Bound by the latency of the row reads (about 1 KB each). With one
 // round, a 16 KiB hash reset per block and half-empty loads of 256 entries a pass, 1,000 queries of 500 candidates
-// took 372 us of a 2.32 ms batch (now 2.13), 500 of 2,000 candidates a fifth of 3.11 ms (now 2.52).
+// took 372 us of a 2.32 ms batch (then 2.13), 500 of 2,000 candidates a fifth of 3.11 ms (then 2.52).
 // Every lane adds its entries (position mod 16 = lane) in order, then the lanes are summed by butterfly: the scores
 // do not depend on the shape.
 __global__ void __launch_bounds__(kRerankThreads) rerank_kernel(RerankArgs a) {
