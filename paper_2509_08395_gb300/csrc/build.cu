@@ -909,12 +909,11 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
         SINDI_CUDA(cudaMemsetAsync(longest, 0, 4, stream));
         longest_list_kernel<<<grid_for(d, 256), 256, 0, stream>>>(ix.seg, d, sigma, longest);
         SINDI_CUDA(cudaGetLastError());
-        if (lp_by_sort(read_u32(longest, stream), Pn, 4 + (dim_bits + 7) / 8)) {
-            uint32_t* inv = P.alloc<uint32_t>(Pn);
-            uint32_t* dcp = P.alloc<uint32_t>(Pn);
-            uint32_t* pos = P.alloc<uint32_t>(Pn);
-            uint32_t* kb = P.alloc<uint32_t>(Pn);
-            uint32_t* db = P.alloc<uint32_t>(Pn);
+        // (the sort's arrays take 20 bytes a posting; without room for them the lists are selected)
+        uint32_t* inv = nullptr;
+        if (lp_by_sort(read_u32(longest, stream), Pn, 4 + (dim_bits + 7) / 8)) inv = P.try_alloc<uint32_t>(5 * Pn);
+        if (inv) {
+            uint32_t *dcp = inv + Pn, *pos = dcp + Pn, *kb = pos + Pn, *db = kb + Pn;
             lp_keys_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(sval, Pn, inv, pos);
             SINDI_CUDA(cudaGetLastError());
             SINDI_CUDA(cudaMemcpyAsync(dcp, sdim, sizeof(uint32_t) * (size_t)Pn, cudaMemcpyDeviceToDevice, stream));
@@ -922,7 +921,7 @@ sindi_status build_lists(IndexImpl& ix, cudaStream_t stream) {
             radix_sort_triples(dcp, inv, pos, kb, db, keep, Pn, dim_bits, P);  // then by dim (stable)
             lp_mark_kernel<<<grid_for(Pn, 256), 256, 0, stream>>>(dcp, pos, Pn, ix.seg, sigma, lp, sdoc, keep, kept);
             SINDI_CUDA(cudaGetLastError());
-            P.free(inv); P.free(dcp); P.free(pos); P.free(kb); P.free(db);
+            P.free(inv);
         } else {
             lp_select_kernel<<<grid_for(d, 1, 152 * 4), kLpBlock, 0, stream>>>(ix.seg, sval, d, sigma, lp, sdoc, keep,
                                                                                kept);
